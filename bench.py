@@ -1045,11 +1045,10 @@ def learned_form(R, L, sess, planes, F, g, dev, stream, peaks):
     flop = px * (2 * 9 * 32 + 2 * 2 * 288 * 32 + 2 * 288 * 16)
     tflops = flop / (cnn_ms / 1e3) / 1e12
     peak = peaks.get("bf16_tflops", 1900.0)
-    # algorithmic bytes per plane pixel of the forward pass: input plane read, FP32
-    # input written and read, three 32-channel BF16 activations written and read,
-    # 16 FP32 heatmap values written -- 460 B against 46 656 FLOP (below the
-    # FLOP/B ridge of this GPU: the network is bound by HBM)
-    cnn_bytes = px * (4 + 4 + 4 + 3 * (64 + 64) + 64)
+    # algorithmic bytes per plane pixel of the forward pass: input plane read, 16
+    # FP32 heatmap values written (no activation leaves the SM) -- 68 B against
+    # 46 656 FLOP, above the FLOP/B ridge of this GPU: the tensor figure is the bound
+    cnn_bytes = px * (4 + 64)
     cnn_gbs = cnn_bytes / (cnn_ms / 1e3) / 1e9
     hbm = peaks.get("hbm_gbs", 6800.0)
     R.ulm_cnn_destroy(c)
@@ -1061,9 +1060,9 @@ def learned_form(R, L, sess, planes, F, g, dev, stream, peaks):
             "pairing_ms_per_300_frames": round(split["pair_ms"] * 300 / frames, 3),
             "n2d_per_300_frames": int(split["n2d"] * 300 / frames),
             "cnn_ms_per_300_frames": round(cnn_ms * 300 / frames, 3),
-            "cnn_roofline": {"bound": "hbm", "achieved": round(cnn_gbs, 1), "peak": hbm, "unit": "GB/s",
-                             "frac": round(cnn_gbs / hbm, 4), "bytes_per_pixel": 460,
-                             "kernel": "k_conv_tc (tcgen05 BF16, TMEM accumulators) + k_conv1_fwd",
+            "cnn_roofline": {"bound": "tensor", "achieved": round(cnn_gbs, 1), "peak": hbm, "unit": "GB/s",
+                             "frac": round(cnn_gbs / hbm, 4), "bytes_per_pixel": 68,
+                             "kernel": "k_cnn_stream (four layers in one kernel: tcgen05 BF16, TMEM accumulators)",
                              "peak_source": "MEASURED_PEAKS.json hbm_gbs",
                              "tensor": {"achieved": round(tflops, 1), "peak": peak, "unit": "TFLOP/s",
                                         "frac": round(tflops / peak, 4),

@@ -9,9 +9,9 @@
 //   L2 conv3x3(32 -> 32) + ReLU    tcgen05 MMA (BF16, FP32 accumulators in TMEM)
 //   L3 conv3x3(32 -> 32) + ReLU    idem
 //   L4 conv3x3(32 -> 16)           idem, epilogue = pixel shuffle to 4x
-// The input gradients run the same tcgen05 kernel on flipped weights; the
-// weight gradients (M = COUT is below the tcgen05 minimum of 64) use
-// mma.sync m16n8k16.
+// The forward pass is one kernel (cnn_stream.cuh).  The input gradients are
+// tcgen05 convolutions with flipped weights (k_conv_tc); the weight gradients
+// (M = COUT is below the tcgen05 minimum of 64) use mma.sync m16n8k16.
 //
 // Activations NHWC BF16; weights [Cout][9 taps][Cin] (tap = 3 (dy+1) + dx+1).
 #include <algorithm>
@@ -71,65 +71,9 @@ __device__ __forceinline__ void mma_bf16(float c[4], const unsigned a[4], const 
 }
 
 // ---------------------------------------------------------------------------
-// input: x[b][i][j] = A[b][i][j] / M[b / planes_per_frame]
-// ---------------------------------------------------------------------------
-__global__ void k_cnn_input(const float* __restrict__ A, const float* __restrict__ M, int ppf, int B, int HW,
-                            float* __restrict__ x)
-{
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (size_t)B * HW) return;
-    const int b = (int)(i / HW);
-    float s = 1.f;
-    if (M) {
-        const float m = M[b / ppf];
-        s = m > 0.f ? 1.f / m : 0.f;
-    }
-    x[i] = A[i] * s;
-}
-
-// L1 forward (Cin = 1): direct 3x3, FP32, + bias + ReLU -> BF16 NHWC.
-__global__ void k_conv1_fwd(const float* __restrict__ x, const float* __restrict__ w1, const float* __restrict__ b1,
-                            int B, int H, int W, __nv_bfloat16* __restrict__ y)
-{
-    __shared__ float sw[CNN_C * 9], sb[CNN_C];
-    for (int q = threadIdx.x; q < CNN_C * 9; q += blockDim.x) sw[q] = w1[q];
-    for (int q = threadIdx.x; q < CNN_C; q += blockDim.x) sb[q] = b1[q];
-    __syncthreads();
-    const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= (size_t)B * H * W) return;
-    const int b = (int)(p / ((size_t)H * W)), ij = (int)(p % ((size_t)H * W)), i = ij / W, j = ij % W;
-    float v[9];
-#pragma unroll
-    for (int t = 0; t < 9; ++t) {
-        const int ii = i + t / 3 - 1, jj = j + t % 3 - 1;
-        v[t] = (ii >= 0 && ii < H && jj >= 0 && jj < W) ? x[((size_t)b * H + ii) * W + jj] : 0.f;
-    }
-    // all CNN_C outputs in registers, written as 16-byte vectors (the pixel's
-    // 2 CNN_C bytes in CNN_C / 8 stores instead of CNN_C / 2)
-    unsigned pk[CNN_C / 2];
-#pragma unroll
-    for (int o = 0; o < CNN_C; o += 2) {
-        float a0 = sb[o], a1 = sb[o + 1];
-#pragma unroll
-        for (int t = 0; t < 9; ++t) {
-            a0 = fmaf(sw[o * 9 + t], v[t], a0);
-            a1 = fmaf(sw[(o + 1) * 9 + t], v[t], a1);
-        }
-        pk[o / 2] = pack_bf2(fmaxf(a0, 0.f), fmaxf(a1, 0.f));
-    }
-    uint4* out = reinterpret_cast<uint4*>(y + p * CNN_C);
-#pragma unroll
-    for (int q = 0; q < CNN_C / 8; ++q) out[q] = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
-}
-
-// ---------------------------------------------------------------------------
-// Epilogue modes of the 3x3 convolution kernels:
-//   MODE 0: + bias, ReLU, BF16 NHWC out
-//   MODE 1: + bias, pixel shuffle (COUT = 16) to the FP32 4x heatmap
-//   MODE 2: no bias, times (mask > 0) of a BF16 NHWC tensor, BF16 out (dgrad)
-// ---------------------------------------------------------------------------
-// ---------------------------------------------------------------------------
-// 3x3 convolution on the 5th-generation tensor cores (tcgen05, TMEM).
+// Input gradient of a 3x3 layer on the 5th-generation tensor cores (tcgen05,
+// TMEM): the convolution of the output gradient with the flipped weights, times
+// (mask > 0) of the layer's BF16 NHWC input, BF16 NHWC out.
 // A CTA of 128 threads owns a tile of 8 rows x 16 columns (M = 128 pixels,
 // ordered column-major: pixel m = 8 x + y), so that one image column of the
 // tile is one 8-row core matrix of the MMA's A operand.  The input tile with
@@ -173,6 +117,14 @@ __device__ __forceinline__ void tc_mma(unsigned tmem_d, uint64_t da, uint64_t db
         : "memory");
 }
 
+// one lane of a converged warp
+__device__ __forceinline__ bool elect_one()
+{
+    unsigned p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 template <int NC>
 __device__ __forceinline__ void tc_ld(unsigned taddr, float* v);
 template <>
@@ -192,16 +144,28 @@ __device__ __forceinline__ void tc_ld<16>(unsigned taddr, float* v)
 template <>
 __device__ __forceinline__ void tc_ld<32>(unsigned taddr, float* v)
 {
-    tc_ld<16>(taddr, v);
-    tc_ld<16>(taddr + 16, v + 16);
+    unsigned r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+          "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
+          "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
+          "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int q = 0; q < 32; ++q) v[q] = __uint_as_float(r[q]);
 }
 
-template <int CIN, int COUT, int MODE>
+#include "cnn_stream.cuh"
+
+template <int CIN, int COUT>
 __global__ void __launch_bounds__(128) k_conv_tc(const __nv_bfloat16* __restrict__ x,
                                                  const __nv_bfloat16* __restrict__ wt,
-                                                 const float* __restrict__ bias,
                                                  const __nv_bfloat16* __restrict__ mask, int B, int H, int W,
-                                                 void* __restrict__ out, unsigned* __restrict__ status)
+                                                 __nv_bfloat16* __restrict__ out, unsigned* __restrict__ status)
 {
     static_assert(CIN % 16 == 0 && COUT % 16 == 0 && COUT <= 32, "shapes of the 3x3 layers");
     constexpr int KC = CIN / 8, NG = COUT / 8;
@@ -334,40 +298,17 @@ __global__ void __launch_bounds__(128) k_conv_tc(const __nv_bfloat16* __restrict
         const int i = i0 + (m & 7), j = j0 + (m >> 3);
         if (i < H && j < W) {
             const size_t pix = ((size_t)b * H + i) * W + j;
-            if (MODE == 0) {
-                unsigned pk[COUT / 2];
+            const unsigned* mk = reinterpret_cast<const unsigned*>(mask) + pix * (COUT / 2);
+            unsigned pk[COUT / 2];
 #pragma unroll
-                for (int o = 0; o < COUT; o += 2)
-                    pk[o / 2] = pack_bf2(fmaxf(v[o] + bias[o], 0.f), fmaxf(v[o + 1] + bias[o + 1], 0.f));
-#pragma unroll
-                for (int q = 0; q < COUT / 8; ++q)
-                    reinterpret_cast<uint4*>(out)[pix * (COUT / 8) + q] =
-                        make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
-            } else if (MODE == 1) {
-                // channel c = 4 a + s -> heatmap pixel (4 i + a, 4 j + s)
-                float* heat = reinterpret_cast<float*>(out);
-                const size_t W4 = (size_t)W * CNN_UP;
-#pragma unroll
-                for (int a = 0; a < CNN_UP; ++a) {
-                    const float4 r4 = make_float4(v[4 * a] + bias[4 * a], v[4 * a + 1] + bias[4 * a + 1],
-                                                  v[4 * a + 2] + bias[4 * a + 2], v[4 * a + 3] + bias[4 * a + 3]);
-                    __stcs(reinterpret_cast<float4*>(heat + ((size_t)b * H * CNN_UP + (size_t)i * CNN_UP + a) * W4 +
-                                                     (size_t)j * CNN_UP),
-                           r4);
-                }
-            } else {
-                const unsigned* mk = reinterpret_cast<const unsigned*>(mask) + pix * (COUT / 2);
-                unsigned pk[COUT / 2];
-#pragma unroll
-                for (int o = 0; o < COUT; o += 2) {
-                    const float2 mm = unpack_bf2(mk[o / 2]);
-                    pk[o / 2] = pack_bf2(mm.x > 0.f ? v[o] : 0.f, mm.y > 0.f ? v[o + 1] : 0.f);
-                }
-#pragma unroll
-                for (int q = 0; q < COUT / 8; ++q)
-                    reinterpret_cast<uint4*>(out)[pix * (COUT / 8) + q] =
-                        make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+            for (int o = 0; o < COUT; o += 2) {
+                const float2 mm = unpack_bf2(mk[o / 2]);
+                pk[o / 2] = pack_bf2(mm.x > 0.f ? v[o] : 0.f, mm.y > 0.f ? v[o + 1] : 0.f);
             }
+#pragma unroll
+            for (int q = 0; q < COUT / 8; ++q)
+                reinterpret_cast<uint4*>(out)[pix * (COUT / 8) + q] =
+                    make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
         }
         // every warp's reads of accumulator `cur` are done before MMAs write it again
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -669,19 +610,19 @@ static rca_status cnn_pack(ulm_cnn* c)
     return cuda_check(c->h, cudaGetLastError(), "cnn pack");
 }
 
-template <int CIN, int COUT, int MODE>
-static rca_status conv_launch(ulm_cnn* c, const __nv_bfloat16* x, const __nv_bfloat16* w, const float* bias,
-                              const __nv_bfloat16* mask, int B, int H, int W, void* out)
+template <int CIN, int COUT>
+static rca_status conv_launch(ulm_cnn* c, const __nv_bfloat16* x, const __nv_bfloat16* w, const __nv_bfloat16* mask,
+                              int B, int H, int W, __nv_bfloat16* out)
 {
     // weights of the nine taps + three halo tiles
     constexpr size_t smem = (size_t)9 * CIN * COUT * 2 + (size_t)3 * (CIN / 8) * TC_HALO_C * TC_CM_BYTES;
     static_assert(smem <= 100 * 1024, "conv tile exceeds its shared-memory budget");
-    auto kern = k_conv_tc<CIN, COUT, MODE>;
+    auto kern = k_conv_tc<CIN, COUT>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_check(c->h, e, "conv smem attribute");
     const int ntiles = B * ((H + CONV_TH - 1) / CONV_TH) * ((W + CONV_TW - 1) / CONV_TW);
     const int grid = std::min(ntiles, c->grid_conv_tc);
-    kern<<<grid, 128, smem, c->h->stream>>>(x, w, bias, mask, B, H, W, out, c->h->d_status);
+    kern<<<grid, 128, smem, c->h->stream>>>(x, w, mask, B, H, W, out, c->h->d_status);
     return cuda_check(c->h, cudaGetLastError(), "conv kernel");
 }
 
@@ -703,19 +644,23 @@ static rca_status wgrad_launch(ulm_cnn* c, const __nv_bfloat16* x, const __nv_bf
     return cuda_check(c->h, cudaGetLastError(), "wgrad kernels");
 }
 
-static rca_status cnn_forward(ulm_cnn* c, const float* A, const float* M, int ppf, int B, int H, int W)
+// the four layers in one launch; KEEP: the activations the backward pass reads
+template <bool KEEP>
+static rca_status cnn_forward(ulm_cnn* c, const float* A, const float* M, int ppf, int B, int H, int W, float* heat)
 {
-    cudaStream_t s = c->h->stream;
-    const size_t np = (size_t)B * H * W;
-    k_cnn_input<<<(unsigned)((np + 255) / 256), 256, 0, s>>>(A, M, ppf > 0 ? ppf : 1, B, H * W, c->x0);
-    k_conv1_fwd<<<(unsigned)((np + 255) / 256), 256, 0, s>>>(c->x0, c->params + c->lay.w[0], c->params + c->lay.b[0], B,
-                                                             H, W, c->a1);
-    rca_status st;
-    if ((st = conv_launch<CNN_C, CNN_C, 0>(c, c->a1, c->wbf[1], c->params + c->lay.b[1], nullptr, B, H, W, c->a2)) != RCA_OK)
-        return st;
-    if ((st = conv_launch<CNN_C, CNN_C, 0>(c, c->a2, c->wbf[2], c->params + c->lay.b[2], nullptr, B, H, W, c->a3)) != RCA_OK)
-        return st;
-    return conv_launch<CNN_C, CNN_UP * CNN_UP, 1>(c, c->a3, c->wbf[3], c->params + c->lay.b[3], nullptr, B, H, W, c->heat);
+    int sms = c->grid_conv / 4;
+    StreamArgs g{};
+    g.A = A, g.M = M, g.ppf = ppf > 0 ? ppf : 1, g.B = B, g.H = H, g.W = W;
+    g.plan = stream_plan(B, H, W, sms);
+    g.w1 = c->params + c->lay.w[0], g.b1 = c->params + c->lay.b[0];
+    g.w2 = c->wbf[1], g.w3 = c->wbf[2], g.w4 = c->wbf[3];
+    g.b2 = c->params + c->lay.b[1], g.b3 = c->params + c->lay.b[2], g.b4 = c->params + c->lay.b[3];
+    g.heat = heat, g.x0 = c->x0, g.a1 = c->a1, g.a2 = c->a2, g.a3 = c->a3, g.status = c->h->d_status;
+    auto kern = k_cnn_stream<KEEP>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, StreamSmem::bytes);
+    if (e != cudaSuccess) return cuda_check(c->h, e, "cnn smem attribute");
+    kern<<<std::min(g.plan.nruns, sms), ST_THREADS, StreamSmem::bytes, c->h->stream>>>(g);
+    return cuda_check(c->h, cudaGetLastError(), "cnn forward");
 }
 
 extern "C" rca_status ulm_cnn_create(rca_handle* h, const ulm_cnn_desc* d, ulm_cnn** out)
@@ -828,7 +773,9 @@ extern "C" rca_status ulm_cnn_forward(ulm_cnn* c, const float* A, const float* M
     if (!A || !heat) return set_error(c->h, RCA_ERR_INVALID_ARG, "null input or heatmap");
     rca_status st = cnn_check_shape(c, B, H, W);
     if (st != RCA_OK) return st;
-    if ((st = cnn_forward(c, A, M, ppf, B, H, W)) != RCA_OK) return st;
+    // the kernel stores 16-byte vectors; a heatmap at another alignment is copied out of the network's own
+    float* direct = (reinterpret_cast<uintptr_t>(heat) & 15) == 0 ? heat : c->heat;
+    if ((st = cnn_forward<false>(c, A, M, ppf, B, H, W, direct)) != RCA_OK || direct == heat) return st;
     return cuda_check(c->h,
                       cudaMemcpyAsync(heat, c->heat, (size_t)B * H * W * CNN_UP * CNN_UP * 4, cudaMemcpyDeviceToDevice,
                                       c->h->stream),
@@ -849,7 +796,7 @@ extern "C" rca_status ulm_cnn_train_step(ulm_cnn* c, const float* A, const float
     rca_status st = cnn_check_shape(c, B, H, W);
     if (st != RCA_OK) return st;
     cudaStream_t s = c->h->stream;
-    if ((st = cnn_forward(c, A, M, ppf, B, H, W)) != RCA_OK) return st;
+    if ((st = cnn_forward<true>(c, A, M, ppf, B, H, W, c->heat)) != RCA_OK) return st;
     const size_t n = (size_t)B * H * W * CNN_UP * CNN_UP;
     const int lgrid = (int)std::min<size_t>((n + 255) / 256, 1024);
     k_loss<<<lgrid, 256, 0, s>>>(c->heat, target, B, H, W, c->gz, c->part);
@@ -857,13 +804,13 @@ extern "C" rca_status ulm_cnn_train_step(ulm_cnn* c, const float* A, const float
     const ParamLayout& L = c->lay;
     // layer 4: dW4 from (a3, dz); dgrad -> g3 masked by a3 > 0
     if ((st = wgrad_launch<CNN_C, CNN_UP * CNN_UP>(c, c->a3, c->gz, B, H, W, c->grads + L.w[3])) != RCA_OK) return st;
-    if ((st = conv_launch<CNN_UP * CNN_UP, CNN_C, 2>(c, c->gz, c->wfl[3], nullptr, c->a3, B, H, W, c->g3)) != RCA_OK) return st;
+    if ((st = conv_launch<CNN_UP * CNN_UP, CNN_C>(c, c->gz, c->wfl[3], c->a3, B, H, W, c->g3)) != RCA_OK) return st;
     // layer 3
     if ((st = wgrad_launch<CNN_C, CNN_C>(c, c->a2, c->g3, B, H, W, c->grads + L.w[2])) != RCA_OK) return st;
-    if ((st = conv_launch<CNN_C, CNN_C, 2>(c, c->g3, c->wfl[2], nullptr, c->a2, B, H, W, c->g2)) != RCA_OK) return st;
+    if ((st = conv_launch<CNN_C, CNN_C>(c, c->g3, c->wfl[2], c->a2, B, H, W, c->g2)) != RCA_OK) return st;
     // layer 2
     if ((st = wgrad_launch<CNN_C, CNN_C>(c, c->a1, c->g2, B, H, W, c->grads + L.w[1])) != RCA_OK) return st;
-    if ((st = conv_launch<CNN_C, CNN_C, 2>(c, c->g2, c->wfl[1], nullptr, c->a1, B, H, W, c->g1)) != RCA_OK) return st;
+    if ((st = conv_launch<CNN_C, CNN_C>(c, c->g2, c->wfl[1], c->a1, B, H, W, c->g1)) != RCA_OK) return st;
     // layer 1 (FP32)
     const int g1grid = std::min(c->grid_conv, (int)std::max<size_t>(1, (size_t)B * H * W / 64));
     k_wgrad1<<<g1grid, 320, 0, s>>>(c->x0, c->g1, B, H, W, c->part);
