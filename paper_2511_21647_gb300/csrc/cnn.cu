@@ -25,6 +25,7 @@
 
 #define CNN_C 32
 #define CNN_UP 4
+#define CNN_LOSS_BLOCKS 1024
 #define CONV_TH 8   // tile rows (one warp each)
 #define CONV_TW 16  // tile columns (the 16 rows of one mma A fragment)
 
@@ -330,190 +331,278 @@ __global__ void __launch_bounds__(128) k_conv_tc(const __nv_bfloat16* __restrict
 // Weight gradient on tensor cores: dW[o][t][c] = sum_p dY[p][o] X[p + t][c],
 // a GEMM with M = COUT, N = 9 x CIN and the reduction over pixels.  Each CTA
 // accumulates its tiles in registers and writes one partial [COUT][9 CIN]
-// (plus the bias partial) to scratch; a second kernel adds the partials in a
-// fixed order (deterministic).  dY and X are staged transposed (channel-major)
-// so that pixel pairs are contiguous for the fragments.
+// (plus the bias partial) to scratch; k_reduce_grads adds the partials in a
+// fixed order (deterministic).  Both operands are reduced over their slow
+// index, so the tiles stay as they lie in memory (pixel-major, 16-byte cp.async
+// copies, two buffers) and ldmatrix transposes them into the fragments; a tap is
+// a shift of whole pixel rows.  One warp per tap; pixel rows are padded by 16
+// bytes, which puts the eight rows of a matrix in different banks.  (With
+// 2-byte transposing stores and gathers: 50 us for 64 planes of 80 x 32, 17 us here.)
 // ---------------------------------------------------------------------------
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(256) k_wgrad_mma(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ dy,
-                                                   int B, int H, int W, float* __restrict__ part)
+#define WG_XS (CNN_C * 2 + 16)                          // bytes of one staged input pixel
+#define WG_DS(COUT) ((COUT) * 2 + 16)                   // of one staged output-gradient pixel
+#define WG_HALO ((CONV_TH + 2) * (CONV_TW + 2))
+#define WG_BUF(COUT) (CONV_TH * CONV_TW * WG_DS(COUT) + WG_HALO * WG_XS)
+
+__device__ __forceinline__ void ldsm_x4_trans(unsigned addr, unsigned r[4])
 {
-    constexpr int TP = CONV_TH * CONV_TW;          // 128 pixels per tile
-    constexpr int DS = TP + 8;                      // dY^T row stride
-    constexpr int HH = CONV_TH + 2, HW2 = CONV_TW + 2;
-    constexpr int XS = HH * HW2 + 8;                // X^T row stride (halo'd tile)
-    constexpr int MT = COUT / 16;                   // m-tiles
-    constexpr int NTT = 9 * CIN / 8;                // n-tiles in total
-    constexpr int NPW = (MT * NTT + 7) / 8;         // (m, n) tiles per warp
-    extern __shared__ __align__(16) unsigned char smraw[];
-    __nv_bfloat16* dYT = reinterpret_cast<__nv_bfloat16*>(smraw);   // [COUT][DS]
-    __nv_bfloat16* XT = dYT + COUT * DS;                            // [CIN][XS]
-    float* dbs = reinterpret_cast<float*>(XT + CIN * XS);           // [COUT]
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+
+__device__ __forceinline__ void cp_async16(unsigned dst, const void* src, bool in)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16u : 0u) : "memory");
+}
+
+template <int COUT>
+__global__ void __launch_bounds__(288, 3) k_wgrad_mma(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ dy,
+                                                      int B, int H, int W, float* __restrict__ part)
+{
+    constexpr int MT = COUT / 16, DC = COUT / 8, DS = WG_DS(COUT), XOFF = CONV_TH * CONV_TW * DS, HW2 = CONV_TW + 2;
+    constexpr int N = 9 * CNN_C;
+    extern __shared__ __align__(16) unsigned char smraw[];   // [2][dY tile, X tile with halo]
+    const int lane = threadIdx.x & 31, tap = threadIdx.x >> 5;
     const int g = lane >> 2, tig = lane & 3;
-    float acc[NPW][4];
+    const unsigned sm = smem_u32(smraw);
+    float acc[MT][4][4], db[MT][2];
 #pragma unroll
-    for (int q = 0; q < NPW; ++q) acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.f;
-    float dbacc = 0.f;  // thread o < COUT accumulates the bias gradient of channel o
+    for (int m = 0; m < MT; ++m) {
+        db[m][0] = db[m][1] = 0.f;
+#pragma unroll
+        for (int n = 0; n < 4; ++n) acc[m][n][0] = acc[m][n][1] = acc[m][n][2] = acc[m][n][3] = 0.f;
+    }
     const int tiles_i = (H + CONV_TH - 1) / CONV_TH, tiles_j = (W + CONV_TW - 1) / CONV_TW;
     const int ntiles = B * tiles_i * tiles_j;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int b = tile / (tiles_i * tiles_j), tij = tile % (tiles_i * tiles_j);
-        const int i0 = (tij / tiles_j) * CONV_TH, j0 = (tij % tiles_j) * CONV_TW;
-        __syncthreads();
-        for (int q = threadIdx.x; q < TP * COUT; q += blockDim.x) {
-            const int p = q / COUT, o = q % COUT;
-            const int ii = i0 + p / CONV_TW, jj = j0 + p % CONV_TW;
-            __nv_bfloat16 v = __float2bfloat16(0.f);
-            if (ii < H && jj < W) v = dy[(((size_t)b * H + ii) * W + jj) * COUT + o];
-            dYT[o * DS + p] = v;
-        }
-        for (int q = threadIdx.x; q < HH * HW2 * CIN; q += blockDim.x) {
-            const int pix = q / CIN, c = q % CIN;
-            const int ii = i0 - 1 + pix / HW2, jj = j0 - 1 + pix % HW2;
-            __nv_bfloat16 v = __float2bfloat16(0.f);
-            if (ii >= 0 && ii < H && jj >= 0 && jj < W) v = x[(((size_t)b * H + ii) * W + jj) * CIN + c];
-            XT[c * XS + pix] = v;
-        }
-        __syncthreads();
-        if (threadIdx.x < COUT) {
-            float s = 0.f;
-            for (int p = 0; p < TP; ++p) s += __bfloat162float(dYT[threadIdx.x * DS + p]);
-            dbacc += s;
-        }
-        // k-steps: each tile row of 16 pixels
-#pragma unroll 1
-        for (int rr = 0; rr < CONV_TH; ++rr) {
-#pragma unroll
-            for (int q = 0; q < NPW; ++q) {
-                const int mn = warp + 8 * q;
-                if (mn >= MT * NTT) break;
-                const int mt = mn % MT, nt = mn / MT;
-                unsigned a[4];
-                const __nv_bfloat16* ya = dYT + (mt * 16 + g) * DS + rr * CONV_TW + 2 * tig;
-                a[0] = *reinterpret_cast<const unsigned*>(ya);
-                a[1] = *reinterpret_cast<const unsigned*>(ya + 8 * DS);
-                a[2] = *reinterpret_cast<const unsigned*>(ya + 8);
-                a[3] = *reinterpret_cast<const unsigned*>(ya + 8 * DS + 8);
-                // column n = nt * 8 + g of N = (tap, cin): tap = n / CIN, c = n % CIN
-                const int n = nt * 8 + g, tap = n / CIN, c = n % CIN;
-                const int dyy = tap / 3, dxx = tap % 3;
-                const __nv_bfloat16* xb = XT + c * XS + (rr + dyy) * HW2 + dxx + 2 * tig;
-                // B(k, n) for pixels k = 2 tig, 2 tig + 1 (and + 8): two bf16 that may be
-                // unaligned in the halo row, so they are gathered as scalars
-                unsigned bb[2];
-                bb[0] = (unsigned)__bfloat16_as_ushort(xb[0]) | ((unsigned)__bfloat16_as_ushort(xb[1]) << 16);
-                bb[1] = (unsigned)__bfloat16_as_ushort(xb[8]) | ((unsigned)__bfloat16_as_ushort(xb[9]) << 16);
-                mma_bf16(acc[q], a, bb);
+    auto load = [&](int tile, int buf) {
+        if (tile < ntiles) {
+            const int b = tile / (tiles_i * tiles_j), tij = tile % (tiles_i * tiles_j);
+            const int i0 = (tij / tiles_j) * CONV_TH, j0 = (tij % tiles_j) * CONV_TW;
+            const unsigned dst = sm + (unsigned)(buf * WG_BUF(COUT));
+            for (int q = threadIdx.x; q < CONV_TH * CONV_TW * DC; q += blockDim.x) {
+                const int c = q % DC, p = q / DC, ii = i0 + p / CONV_TW, jj = j0 + p % CONV_TW;
+                const bool in = ii < H && jj < W;
+                cp_async16(dst + p * DS + c * 16, in ? dy + (((size_t)b * H + ii) * W + jj) * COUT + c * 8 : dy, in);
+            }
+            for (int q = threadIdx.x; q < WG_HALO * (CNN_C / 8); q += blockDim.x) {
+                const int c = q % (CNN_C / 8), p = q / (CNN_C / 8), ii = i0 - 1 + p / HW2, jj = j0 - 1 + p % HW2;
+                const bool in = ii >= 0 && ii < H && jj >= 0 && jj < W;
+                cp_async16(dst + XOFF + p * WG_XS + c * 16, in ? x + (((size_t)b * H + ii) * W + jj) * CNN_C + c * 8 : x, in);
             }
         }
-    }
-    // partial of this CTA: rows (o) g, g + 8 of m-tile, columns n = nt*8 + 2 tig (+1)
-    float* dst = part + (size_t)blockIdx.x * (COUT * 9 * CIN + COUT);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // fragment addresses of this lane: dY (pixel, 8-output chunk) and X (pixel, 8-channel chunk)
+    const unsigned la = (unsigned)(((lane >> 4) * 8 + (lane & 7)) * DS + (lane >> 3 & 1) * 16);
+    const unsigned lb = (unsigned)(XOFF + ((tap / 3) * HW2 + tap % 3 + (lane >> 3 & 1) * 8 + (lane & 7)) * WG_XS +
+                                   (lane >> 4) * 16);
+    int buf = 0;
+    load(blockIdx.x, 0);
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, buf ^= 1) {
+        load(tile + gridDim.x, buf ^ 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();
+        const unsigned base = sm + (unsigned)(buf * WG_BUF(COUT));
+#pragma unroll 2
+        for (int rr = 0; rr < CONV_TH; ++rr) {                 // k-steps: the 16 pixels of a tile row
+            unsigned a[MT][4], bb[2][4];
 #pragma unroll
-    for (int q = 0; q < NPW; ++q) {
-        const int mn = warp + 8 * q;
-        if (mn >= MT * NTT) break;
-        const int mt = mn % MT, nt = mn / MT;
-        const int o0 = mt * 16 + g, n0 = nt * 8 + 2 * tig;
-        dst[o0 * 9 * CIN + n0] = acc[q][0];
-        dst[o0 * 9 * CIN + n0 + 1] = acc[q][1];
-        dst[(o0 + 8) * 9 * CIN + n0] = acc[q][2];
-        dst[(o0 + 8) * 9 * CIN + n0 + 1] = acc[q][3];
+            for (int m = 0; m < MT; ++m) ldsm_x4_trans(base + la + rr * CONV_TW * DS + m * 32, a[m]);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) ldsm_x4_trans(base + lb + rr * HW2 * WG_XS + j * 32, bb[j]);
+#pragma unroll
+            for (int m = 0; m < MT; ++m)
+#pragma unroll
+                for (int n = 0; n < 4; ++n) mma_bf16(acc[m][n], a[m], bb[n >> 1] + 2 * (n & 1));
+            if (tap == 0) {
+#pragma unroll
+                for (int m = 0; m < MT; ++m)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float2 v = unpack_bf2(a[m][q]);
+                        db[m][q & 1] += v.x + v.y;
+                    }
+            }
+        }
+        __syncthreads();                                       // the buffer is filled again two tiles on
     }
-    (void)dbs;
-    if (threadIdx.x < COUT) dst[COUT * 9 * CIN + threadIdx.x] = dbacc;
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    // partial of this CTA: rows (o) g, g + 8 of each m-tile, columns tap * 32 + n * 8 + 2 tig (+1)
+    float* dst = part + (size_t)blockIdx.x * (COUT * N + COUT);
+#pragma unroll
+    for (int m = 0; m < MT; ++m)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int o = m * 16 + g + 8 * h;
+#pragma unroll
+            for (int n = 0; n < 4; ++n)
+                *reinterpret_cast<float2*>(dst + o * N + tap * CNN_C + n * 8 + 2 * tig) =
+                    make_float2(acc[m][n][2 * h], acc[m][n][2 * h + 1]);
+            float s = db[m][h];
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            if (tap == 0 && tig == 0) dst[COUT * N + o] = s;
+        }
 }
 
-// L1 weight gradient (CIN = 1), FP32: per-CTA partials of dW1[o][t], db1[o].
-__global__ void k_wgrad1(const float* __restrict__ x, const __nv_bfloat16* __restrict__ dy, int B, int H, int W,
-                         float* __restrict__ part)
+// L1 weight gradient (CIN = 1), FP32: per-CTA partials of dW1[o][t], db1[o].  A
+// warp walks one plane row, its lanes being the 32 output channels: one 64-byte
+// load of the output gradient and three broadcast loads of the input per pixel
+// feed ten sums in registers.  (With a thread per (o, t) and one pixel at a
+// time: 288 us for 64 planes of 80 x 32, 14 us here.)
+__global__ void __launch_bounds__(256) k_wgrad1(const float* __restrict__ x, const __nv_bfloat16* __restrict__ dy, int rows,
+                                                int H, int W, float* __restrict__ part)
 {
-    // thread (o, t) for o < 32, t < 10 (t = 9: bias); CTA strides over pixels
-    __shared__ float red[CNN_C * 10];
-    const int o = threadIdx.x / 10, t = threadIdx.x % 10;
-    float s = 0.f;
-    if (threadIdx.x < CNN_C * 10) {
-        const size_t np = (size_t)B * H * W;
-        for (size_t p = blockIdx.x; p < np; p += gridDim.x) {
-            const int b = (int)(p / ((size_t)H * W)), ij = (int)(p % ((size_t)H * W)), i = ij / W, j = ij % W;
-            const float d = __bfloat162float(dy[p * CNN_C + o]);
-            if (t == 9) {
-                s += d;
-            } else {
-                const int ii = i + t / 3 - 1, jj = j + t % 3 - 1;
-                if (ii >= 0 && ii < H && jj >= 0 && jj < W) s = fmaf(d, x[((size_t)b * H + ii) * W + jj], s);
-            }
+    __shared__ float red[8][CNN_C * 10];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float s[10];
+#pragma unroll
+    for (int t = 0; t < 10; ++t) s[t] = 0.f;
+    for (int r = blockIdx.x * 8 + warp; r < rows; r += gridDim.x * 8) {
+        const int i = r % H;
+        const float* xr = x + (size_t)r * W;
+        const __nv_bfloat16* dr = dy + (size_t)r * W * CNN_C + lane;
+        const bool up = i > 0, dn = i + 1 < H;
+        float v[3][3];                                         // [row][column j - 1, j, j + 1]
+#pragma unroll
+        for (int q = 0; q < 3; ++q) v[q][0] = v[q][1] = 0.f;
+        v[0][2] = up ? xr[-W] : 0.f, v[1][2] = xr[0], v[2][2] = dn ? xr[W] : 0.f;
+#pragma unroll 4
+        for (int j = 0; j < W; ++j) {
+            const bool in = j + 1 < W;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) v[q][0] = v[q][1], v[q][1] = v[q][2];
+            v[0][2] = up && in ? xr[j + 1 - W] : 0.f;
+            v[1][2] = in ? xr[j + 1] : 0.f;
+            v[2][2] = dn && in ? xr[j + 1 + W] : 0.f;
+            const float d = __bfloat162float(dr[(size_t)j * CNN_C]);
+#pragma unroll
+            for (int t = 0; t < 9; ++t) s[t] = fmaf(d, v[t / 3][t % 3], s[t]);
+            s[9] += d;
         }
-        red[threadIdx.x] = s;
     }
+#pragma unroll
+    for (int t = 0; t < 10; ++t) red[warp][t < 9 ? lane * 9 + t : CNN_C * 9 + lane] = s[t];
     __syncthreads();
-    if (threadIdx.x < CNN_C * 10) {
-        float* dst = part + (size_t)blockIdx.x * (CNN_C * 9 + CNN_C);
-        if (t < 9) dst[o * 9 + t] = red[threadIdx.x];
-        else dst[CNN_C * 9 + o] = red[threadIdx.x];
+    for (int k = threadIdx.x; k < CNN_C * 10; k += 256) {
+        float t = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) t += red[w][k];
+        part[(size_t)blockIdx.x * (CNN_C * 10) + k] = t;
     }
 }
 
-// sum CTA partials in a fixed order: out[k] = sum_c part[c][k]
-__global__ void k_reduce_partials(const float* __restrict__ part, int nparts, int len, float* __restrict__ out)
+// Sums of the CTAs' partials in a fixed order: every layer's gradients and the
+// loss in one launch.  A block adds 32 columns, eight warps taking every
+// eighth partial, so that a column's loads are not one serial chain (four launches
+// of one thread per column: 157 us for 608 partials, 8 us here).
+struct GradSums {
+    const float* part[5];
+    int nparts[5], len[5], block0[6];   // layers 1..4, then the loss (one column); first block of each
+    float* out[5];
+    float scale[5];
+};
+
+__global__ void __launch_bounds__(256) k_reduce_grads(const GradSums g)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= len) return;
+    __shared__ float red[8][32];
+    int seg = 0;
+    while (seg < 4 && (int)blockIdx.x >= g.block0[seg + 1]) ++seg;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int len = g.len[seg], np = g.nparts[seg], k = ((int)blockIdx.x - g.block0[seg]) * 32 + lane;
+    const float* p = g.part[seg];
     float s = 0.f;
-    for (int c = 0; c < nparts; ++c) s += part[(size_t)c * len + k];
-    out[k] = s;
+    if (seg == 4) {                                            // one column: spread its partials over the block
+        for (int c = threadIdx.x; c < np; c += 256) s += p[c];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    } else if (k < len) {
+#pragma unroll 8
+        for (int c = warp; c < np; c += 8) s += p[(size_t)c * len + k];
+    }
+    red[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0 && k < len) {
+        float t = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) t += red[w][lane];
+        g.out[seg][k] = t * g.scale[seg];
+    }
 }
 
 // MSE loss: per-CTA partial sums of (heat - target)^2 and dZ4 (un-shuffled
-// 2 (heat - target) / n, BF16 NHWC with 16 channels).
-__global__ void k_loss(const float* __restrict__ heat, const float* __restrict__ target, int B, int H, int W,
-                       __nv_bfloat16* __restrict__ dz, float* __restrict__ part)
+// 2 (heat - target) / n, BF16 NHWC with 16 channels).  A thread owns one plane
+// pixel: four 16-byte runs of the heatmap and of the target, one 32-byte gradient
+// (element by element with its divisions: 18 us for 64 planes of 80 x 32, 6 us here).
+template <bool ALIGNED>
+__global__ void __launch_bounds__(256) k_loss(const float* __restrict__ heat, const float* __restrict__ target, int rows,
+                                              int W, float scale, __nv_bfloat16* __restrict__ dz, float* __restrict__ part)
 {
-    __shared__ float red[32];
-    const size_t n = (size_t)B * H * W * CNN_UP * CNN_UP;
-    const float scale = 2.0f / (float)n;
+    __shared__ float red[8];
+    const unsigned np = (unsigned)rows * W;                    // within the network's capacity, an int
     float s = 0.f;
-    for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (size_t)gridDim.x * blockDim.x) {
-        const size_t W4 = (size_t)W * CNN_UP;
-        const size_t b = q / ((size_t)H * CNN_UP * W4), rem = q % ((size_t)H * CNN_UP * W4);
-        const int y = (int)(rem / W4), xq = (int)(rem % W4);
-        const float d = heat[q] - target[q];
-        s = fmaf(d, d, s);
-        const int i = y / CNN_UP, a = y % CNN_UP, j = xq / CNN_UP, c = xq % CNN_UP;
-        dz[(((b * H + i) * W + j) * (CNN_UP * CNN_UP)) + a * CNN_UP + c] = __float2bfloat16(d * scale);
+    for (unsigned p = blockIdx.x * 256 + threadIdx.x; p < np; p += gridDim.x * 256) {
+        const unsigned r = p / W, j = p - r * W;
+        const size_t at = ((size_t)r * CNN_UP * W + j) * CNN_UP;
+        float4 h[CNN_UP], t[CNN_UP];
+#pragma unroll
+        for (int a = 0; a < CNN_UP; ++a) {
+            const size_t q = at + (size_t)a * W * CNN_UP;
+            h[a] = __ldg(reinterpret_cast<const float4*>(heat + q));
+            t[a] = ALIGNED ? __ldg(reinterpret_cast<const float4*>(target + q))
+                           : make_float4(target[q], target[q + 1], target[q + 2], target[q + 3]);
+        }
+        unsigned pk[2 * CNN_UP];
+#pragma unroll
+        for (int a = 0; a < CNN_UP; ++a) {
+            const float d0 = h[a].x - t[a].x, d1 = h[a].y - t[a].y, d2 = h[a].z - t[a].z, d3 = h[a].w - t[a].w;
+            s = fmaf(d0, d0, s), s = fmaf(d1, d1, s), s = fmaf(d2, d2, s), s = fmaf(d3, d3, s);
+            pk[2 * a] = pack_bf2(d0 * scale, d1 * scale);
+            pk[2 * a + 1] = pack_bf2(d2 * scale, d3 * scale);
+        }
+        uint4* o = reinterpret_cast<uint4*>(dz + (size_t)p * (CNN_UP * CNN_UP));
+        o[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        o[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
         float t = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
+        for (int w = 0; w < 8; ++w) t += red[w];
         part[blockIdx.x] = t;
     }
 }
 
-__global__ void k_loss_final(const float* __restrict__ part, int nparts, float inv_n, float* __restrict__ loss)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        float s = 0.f;
-        for (int c = 0; c < nparts; ++c) s += part[c];
-        *loss = s * inv_n;
-    }
-}
+// Adam on the FP32 masters (bias-corrected step sizes computed on the host),
+// then the BF16 copies of the updated weights (as k_pack_weights)
+struct PackedWeights {
+    ParamLayout lay;
+    __nv_bfloat16 *fwd[4], *flip[4];
+};
 
-// Adam on the FP32 masters (bias-corrected step sizes computed on the host)
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ gr, float* __restrict__ m, float* __restrict__ v,
-                       int n, float lr_t, float b1, float b2, float eps_t)
+                       const PackedWeights w, float lr_t, float b1, float b2, float eps_t)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= w.lay.total) return;
     const float g = gr[i];
     const float mi = b1 * m[i] + (1.f - b1) * g;
     const float vi = b2 * v[i] + (1.f - b2) * g * g;
     m[i] = mi;
     v[i] = vi;
-    p[i] -= lr_t * mi / (sqrtf(vi) + eps_t);
+    const float pn = p[i] - lr_t * mi / (sqrtf(vi) + eps_t);
+    p[i] = pn;
+#pragma unroll
+    for (int l = 1; l < 4; ++l) {
+        const int q = i - w.lay.w[l], O = l == 3 ? CNN_UP * CNN_UP : CNN_C;
+        if (q < 0 || q >= O * 9 * CNN_C) continue;
+        const int o = q / (9 * CNN_C), t = (q / CNN_C) % 9, c = q % CNN_C;
+        const __nv_bfloat16 h = __float2bfloat16(pn);
+        w.fwd[l][q] = h;
+        w.flip[l][((size_t)c * 9 + (8 - t)) * O + o] = h;
+    }
 }
 
 // BF16 copies of the weights: forward layout [O][9][I] and, for the input
@@ -586,8 +675,9 @@ struct ulm_cnn {
     float* heat = nullptr;
     float* part = nullptr;  // scratch for per-CTA partials
     size_t part_len = 0;
-    int grid_conv = 0;
-    int grid_conv_tc = 0;
+    int sms = 0;
+    int grid_conv_tc = 0;   // input-gradient CTAs: four per SM (64 TMEM columns each)
+    int grid_wgrad = 0;     // weight-gradient CTAs, each with one partial: three per SM
 };
 
 static rca_status cnn_check_shape(ulm_cnn* c, int B, int H, int W)
@@ -626,29 +716,27 @@ static rca_status conv_launch(ulm_cnn* c, const __nv_bfloat16* x, const __nv_bfl
     return cuda_check(c->h, cudaGetLastError(), "conv kernel");
 }
 
-template <int CIN, int COUT>
-static rca_status wgrad_launch(ulm_cnn* c, const __nv_bfloat16* x, const __nv_bfloat16* dy, int B, int H, int W,
-                               float* dw)
+// weight gradient partials of layer l + 1 into their part of the scratch
+template <int COUT>
+static rca_status wgrad_launch(ulm_cnn* c, const __nv_bfloat16* x, const __nv_bfloat16* dy, int B, int H, int W, int l,
+                               GradSums& sums, size_t& at)
 {
-    constexpr int DS = CONV_TH * CONV_TW + 8, XS = (CONV_TH + 2) * (CONV_TW + 2) + 8;
-    const size_t smem = ((size_t)COUT * DS + (size_t)CIN * XS) * sizeof(__nv_bfloat16) + COUT * sizeof(float);
-    auto kern = k_wgrad_mma<CIN, COUT>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kern = k_wgrad_mma<COUT>;
+    const int smem = 2 * WG_BUF(COUT);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return cuda_check(c->h, e, "wgrad smem attribute");
     const int ntiles = B * ((H + CONV_TH - 1) / CONV_TH) * ((W + CONV_TW - 1) / CONV_TW);
-    const int grid = std::min(ntiles, c->grid_conv);
-    const int len = COUT * 9 * CIN + COUT;
-    if ((size_t)grid * len > c->part_len) return set_error(c->h, RCA_ERR_CAPACITY, "cnn scratch too small");
-    kern<<<grid, 256, smem, c->h->stream>>>(x, dy, B, H, W, c->part);
-    k_reduce_partials<<<(len + 255) / 256, 256, 0, c->h->stream>>>(c->part, grid, len, dw);
-    return cuda_check(c->h, cudaGetLastError(), "wgrad kernels");
+    sums.part[l] = c->part + at, sums.nparts[l] = std::min(ntiles, c->grid_wgrad), sums.len[l] = COUT * 9 * CNN_C + COUT;
+    kern<<<sums.nparts[l], 288, smem, c->h->stream>>>(x, dy, B, H, W, c->part + at);
+    at += (size_t)c->grid_wgrad * sums.len[l];
+    return cuda_check(c->h, cudaGetLastError(), "wgrad kernel");
 }
 
 // the four layers in one launch; KEEP: the activations the backward pass reads
 template <bool KEEP>
 static rca_status cnn_forward(ulm_cnn* c, const float* A, const float* M, int ppf, int B, int H, int W, float* heat)
 {
-    int sms = c->grid_conv / 4;
+    const int sms = c->sms;
     StreamArgs g{};
     g.A = A, g.M = M, g.ppf = ppf > 0 ? ppf : 1, g.B = B, g.H = H, g.W = W;
     g.plan = stream_plan(B, H, W, sms);
@@ -679,9 +767,12 @@ extern "C" rca_status ulm_cnn_create(rca_handle* h, const ulm_cnn_desc* d, ulm_c
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    c->grid_conv = 4 * sms;
-    c->grid_conv_tc = 4 * sms;   // four CTAs per SM (64 TMEM columns each)
-    c->part_len = (size_t)c->grid_conv * (CNN_C * 9 * CNN_C + CNN_C) + 4096;
+    c->sms = sms;
+    c->grid_conv_tc = 4 * sms;
+    c->grid_wgrad = 3 * sms;
+    // partials of layers 4, 3, 2 and 1, then of the loss
+    c->part_len = (size_t)c->grid_wgrad * (CNN_UP * CNN_UP * (9 * CNN_C + 1) + 2 * CNN_C * (9 * CNN_C + 1) + CNN_C * 10) +
+                  CNN_LOSS_BLOCKS;
     const size_t P = c->lay.total, px = c->cap_px;
     bool ok = cudaMalloc(&c->params, P * 4) == cudaSuccess && cudaMalloc(&c->grads, P * 4) == cudaSuccess &&
               cudaMalloc(&c->m, P * 4) == cudaSuccess && cudaMalloc(&c->v, P * 4) == cudaSuccess &&
@@ -797,24 +888,34 @@ extern "C" rca_status ulm_cnn_train_step(ulm_cnn* c, const float* A, const float
     if (st != RCA_OK) return st;
     cudaStream_t s = c->h->stream;
     if ((st = cnn_forward<true>(c, A, M, ppf, B, H, W, c->heat)) != RCA_OK) return st;
-    const size_t n = (size_t)B * H * W * CNN_UP * CNN_UP;
-    const int lgrid = (int)std::min<size_t>((n + 255) / 256, 1024);
-    k_loss<<<lgrid, 256, 0, s>>>(c->heat, target, B, H, W, c->gz, c->part);
-    k_loss_final<<<1, 32, 0, s>>>(c->part, lgrid, 1.0f / (float)n, loss_dev);
     const ParamLayout& L = c->lay;
+    const size_t px = (size_t)B * H * W;
+    const float n = (float)(px * CNN_UP * CNN_UP);
+    GradSums sums{};
+    size_t at = 0;
+    const int lgrid = (int)std::min<size_t>((px + 255) / 256, CNN_LOSS_BLOCKS);
+    float* lpart = c->part + (c->part_len - CNN_LOSS_BLOCKS);
+    if ((reinterpret_cast<uintptr_t>(target) & 15) == 0)
+        k_loss<true><<<lgrid, 256, 0, s>>>(c->heat, target, B * H, W, 2.0f / n, c->gz, lpart);
+    else
+        k_loss<false><<<lgrid, 256, 0, s>>>(c->heat, target, B * H, W, 2.0f / n, c->gz, lpart);
     // layer 4: dW4 from (a3, dz); dgrad -> g3 masked by a3 > 0
-    if ((st = wgrad_launch<CNN_C, CNN_UP * CNN_UP>(c, c->a3, c->gz, B, H, W, c->grads + L.w[3])) != RCA_OK) return st;
+    if ((st = wgrad_launch<CNN_UP * CNN_UP>(c, c->a3, c->gz, B, H, W, 3, sums, at)) != RCA_OK) return st;
     if ((st = conv_launch<CNN_UP * CNN_UP, CNN_C>(c, c->gz, c->wfl[3], c->a3, B, H, W, c->g3)) != RCA_OK) return st;
     // layer 3
-    if ((st = wgrad_launch<CNN_C, CNN_C>(c, c->a2, c->g3, B, H, W, c->grads + L.w[2])) != RCA_OK) return st;
+    if ((st = wgrad_launch<CNN_C>(c, c->a2, c->g3, B, H, W, 2, sums, at)) != RCA_OK) return st;
     if ((st = conv_launch<CNN_C, CNN_C>(c, c->g3, c->wfl[2], c->a2, B, H, W, c->g2)) != RCA_OK) return st;
     // layer 2
-    if ((st = wgrad_launch<CNN_C, CNN_C>(c, c->a1, c->g2, B, H, W, c->grads + L.w[1])) != RCA_OK) return st;
+    if ((st = wgrad_launch<CNN_C>(c, c->a1, c->g2, B, H, W, 1, sums, at)) != RCA_OK) return st;
     if ((st = conv_launch<CNN_C, CNN_C>(c, c->g2, c->wfl[1], c->a1, B, H, W, c->g1)) != RCA_OK) return st;
     // layer 1 (FP32)
-    const int g1grid = std::min(c->grid_conv, (int)std::max<size_t>(1, (size_t)B * H * W / 64));
-    k_wgrad1<<<g1grid, 320, 0, s>>>(c->x0, c->g1, B, H, W, c->part);
-    k_reduce_partials<<<(CNN_C * 10 + 255) / 256, 256, 0, s>>>(c->part, g1grid, CNN_C * 10, c->grads + L.w[0]);
+    sums.part[0] = c->part + at, sums.nparts[0] = std::min(c->grid_wgrad, (B * H + 7) / 8), sums.len[0] = CNN_C * 10;
+    k_wgrad1<<<sums.nparts[0], 256, 0, s>>>(c->x0, c->g1, B * H, H, W, c->part + at);
+    // every layer's sums and the loss
+    sums.part[4] = lpart, sums.nparts[4] = lgrid, sums.len[4] = 1, sums.out[4] = loss_dev, sums.scale[4] = 1.0f / n;
+    for (int l = 0; l < 4; ++l) sums.out[l] = c->grads + L.w[l], sums.scale[l] = 1.f;
+    for (int l = 0; l < 5; ++l) sums.block0[l + 1] = sums.block0[l] + (sums.len[l] + 31) / 32;
+    k_reduce_grads<<<sums.block0[5], 256, 0, s>>>(sums);
     if ((st = cuda_check(c->h, cudaGetLastError(), "backward kernels")) != RCA_OK) return st;
     if (!apply_update) return RCA_OK;
     c->step += 1;
@@ -823,10 +924,11 @@ extern "C" rca_status ulm_cnn_train_step(ulm_cnn* c, const float* A, const float
     // p -= lr * (m / bc1) / (sqrt(v / bc2) + eps)  ==  lr_t * m / (sqrt(v) + eps_t)
     const float lr_t = (float)(c->desc.lr * std::sqrt(bc2) / bc1);
     const float eps_t = (float)(c->desc.eps * std::sqrt(bc2));
-    k_adam<<<(L.total + 255) / 256, 256, 0, s>>>(c->params, c->grads, c->m, c->v, L.total, lr_t, (float)b1, (float)b2,
-                                                eps_t);
-    if ((st = cuda_check(c->h, cudaGetLastError(), "adam")) != RCA_OK) return st;
-    return cnn_pack(c);
+    PackedWeights w{};
+    w.lay = L;
+    for (int l = 1; l < 4; ++l) w.fwd[l] = c->wbf[l], w.flip[l] = c->wfl[l];
+    k_adam<<<(L.total + 255) / 256, 256, 0, s>>>(c->params, c->grads, c->m, c->v, w, lr_t, (float)b1, (float)b2, eps_t);
+    return cuda_check(c->h, cudaGetLastError(), "adam");
 }
 
 extern "C" rca_status ulm_cnn_target(rca_handle* h, const float* pts, int n, int B, int H4, int W4, float sigma,
