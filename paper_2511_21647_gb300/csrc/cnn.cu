@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(256) k_wgrad1(const float* __restrict__ x, con
 // Sums of the CTAs' partials in a fixed order: every layer's gradients and the
 // loss in one launch.  A block adds 32 columns, eight warps taking every
 // eighth partial, so that a column's loads are not one serial chain (four launches
-// of one thread per column: 157 us for 608 partials, 8 us here).
+// of one thread per column, 608 partials: 157 us; 456 partials here: 10 us).
 struct GradSums {
     const float* part[5];
     int nparts[5], len[5], block0[6];   // layers 1..4, then the loss (one column); first block of each
