@@ -510,7 +510,7 @@ extern "C" rca_status ulm_pair3d(rca_handle* h, const rca_tables* t, const ulm_l
     if (!n2d || !n3d || cap2d < 0 || cap3d < 0 || (cap2d > 0 && !L) || (cap3d > 0 && !out))
         return set_error(h, RCA_ERR_INVALID_ARG, "null list or count");
     DeviceGuard dg(h->device);
-    return launch_pair3d(h, t, L, n2d, cap2d, F, out, cap3d, n3d);
+    return launch_pair3d(h, t, L, n2d, cap2d, F, out, cap3d, n3d, nullptr);
 }
 
 extern "C" rca_status ulm_pair3d_noalloc(rca_handle* h, const rca_tables* t, const ulm_loc2d* L, const int* n2d,
@@ -659,8 +659,7 @@ extern "C" rca_status ulm_localize(rca_handle* h, const rca_tables* t, const voi
     float* M = (float*)ws_get(h, WS_M, (size_t)F * sizeof(float), &st);
     if (!M) return st;
     if ((st = launch_enhance(h, t, planes, pt, F, prm->enh, A, M)) != RCA_OK) return st;
-    if ((st = launch_detect2d(h, t, A, M, F, prm, out2d, cap2d, n2d, nullptr, nullptr)) != RCA_OK) return st;
-    return launch_pair3d(h, t, out2d, n2d, cap2d, F, out3d, cap3d, n3d);
+    return launch_detect_pair(h, t, A, M, F, prm, out2d, cap2d, n2d, out3d, cap3d, n3d);
 }
 
 extern "C" rca_status ulm_detect_map(rca_handle* h, const rca_tables* t, const float* map, int up, const float* A,
@@ -973,10 +972,8 @@ static rca_status batch_enqueue(rca_batch* b)
         st = cuda_check(b->h, cudaStreamWaitEvent(h->stream, b->bf_done, 0), "batch fork wait");
         if (st == RCA_OK) st = launch_enhance(h, t, b->ens[e].planes, b->pl_t, F, b->prm.enh, b->A[e], b->M[e]);
         if (st == RCA_OK)
-            st = launch_detect2d(h, t, b->A[e], b->M[e], F, &b->prm, b->out2d[e], b->cap2d[e], b->n2d[e], nullptr,
-                                 nullptr);
-        if (st == RCA_OK)
-            st = launch_pair3d(h, t, b->out2d[e], b->n2d[e], b->cap2d[e], F, b->out3d[e], b->cap3d[e], b->n3d[e]);
+            st = launch_detect_pair(h, t, b->A[e], b->M[e], F, &b->prm, b->out2d[e], b->cap2d[e], b->n2d[e], b->out3d[e],
+                                    b->cap3d[e], b->n3d[e]);
         if (!h->last_error.empty()) b->h->last_error = h->last_error;
         // join (also after a failed launch, so a capture stays well formed)
         cudaEventRecord(b->ldone[e], h->stream);

@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(256) k_enhance(const void* __restrict__ planes
 // consecutive row pairs (row-pair stride of N + 1 pairs) in the horizontal
 // pass.
 // ---------------------------------------------------------------------------
-#define NCC_THREADS 256
+#define NCC_THREADS 256   // 128 for planes of up to 64 columns, whose passes have no more tasks
 
 // float2 columns of one padded vertical-sum row pair (see k_detect)
 __host__ __device__ inline int det_npad(int N, int H, int HB)
@@ -147,10 +147,49 @@ __device__ __forceinline__ void split_box(LOAD in, uint64_t (&out)[NB])
     }
 }
 
-template <int H, int NC>
-__global__ void __launch_bounds__(NCC_THREADS, 2) k_detect(const float* __restrict__ A, const float* __restrict__ Mf,
+// the count of candidate slot s: kept in full, added to the kept total of its
+// chunk of GATHER_SLOTS slots (for the gather's offsets) and to the true total
+#define GATHER_SLOTS 256
+__device__ __forceinline__ void slot_count(int* __restrict__ cnt, int* __restrict__ part,
+                                           unsigned long long* __restrict__ total, int s, int n, unsigned* __restrict__ status)
+{
+    cnt[s] = n;
+    if (n > 0) {
+        atomicAdd(part + s / GATHER_SLOTS, min(n, CAND_CAP));
+        atomicAdd(total, (unsigned long long)n);
+    }
+    if (n > CAND_CAP) atomicOr(status, ST_CAPACITY);
+}
+
+// Whether NCC row ro, column l of the NCC rows sN is a 3 x 3 regional maximum.
+__device__ __forceinline__ bool ncc_peak(const float* __restrict__ sN, int NS, int ro, int l)
+{
+    const float c = sN[ro * NS + l];
+    bool pk = true;
+#pragma unroll
+    for (int a = -1; a <= 1; ++a)
+#pragma unroll
+        for (int b = -1; b <= 1; ++b) {
+            if (a == 0 && b == 0) continue;
+            const float v = sN[(ro + a) * NS + l + b];
+            const bool earlier = (a < 0) || (a == 0 && b < 0);
+            pk = pk && (earlier ? (c > v) : (c >= v));
+        }
+    return pk;
+}
+
+// NT threads run the two correlation passes; one warp more serves them: it fetches
+// the strips, and while the others are at the next strip it tests the last one's
+// few pixels over the thresholds and writes the peaks.  (With all threads walking
+// the pixels for peaks, compacting and fetching between barriers, the paper's 300
+// frames at d = 11 took 1.40 ms, now 1.18.)  What is left is the two passes: issue
+// slots half used, the barriers after either pass the largest stall.
+#define DET_LIST 1024   // pixels over the thresholds that the serving warp takes; beyond, all threads test
+template <int H, int NC, int NT>
+__global__ void __launch_bounds__(NT + 32, 512 / NT) k_detect(const float* __restrict__ A, const float* __restrict__ Mf,
                                                           int S, int nz, int Nrt, int nplanes, NccConst nc,
                                                           ulm_loc2d* __restrict__ cand, int* __restrict__ cnt,
+                                                          int* __restrict__ part, unsigned long long* __restrict__ total,
                                                           float* __restrict__ ncc_out, unsigned* __restrict__ status)
 {
     constexpr int D = 2 * H + 1;
@@ -174,16 +213,25 @@ __global__ void __launch_bounds__(NCC_THREADS, 2) k_detect(const float* __restri
     // sm + bb abuf (bb = 0, 1): [rin][N] amplitude rows i0-1-H ..., double-buffered
     float* sV = sm + 2 * abuf;              // [3][RP][NPAD][2]; column c at c + H
     // [RN][N] flags A >= alpha M_t of the NCC rows' pixels, set by the vertical pass
-    // (which holds the amplitudes), so that no phase after it reads global memory
+    // (which holds the amplitudes), so that the horizontal pass reads no global memory
     unsigned char* aflag = reinterpret_cast<unsigned char*>(sV + (size_t)3 * RP * NPAD * 2);
-    __shared__ unsigned bits[NW];           // candidate pixels of the strip, raster order
-    __shared__ int wsum[NCC_THREADS / 32];
-    __shared__ uint64_t bar[2];
+    // of the items of either buffer: the pixels with NCC >= ncc_min and their flag set,
+    // in no order; their peaks, in raster order
+    __shared__ unsigned short list[2][DET_LIST];
+    __shared__ unsigned bits[2][NW];
+    __shared__ unsigned short order[CAND_CAP];
+    __shared__ int nlist[2];
+    __shared__ uint64_t full[2], done[2];   // rows fetched; NCC rows and list complete
+    const int nwords = (NCC_RS * N + 31) / 32;
     if (threadIdx.x == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
+        for (int q = 0; q < 2; ++q) {
+            mbar_init(&full[q], 1);
+            mbar_init(&done[q], NT / 32);   // one arrival per warp: an arrival is a serialised access
+            nlist[q] = 0;
+        }
         mbar_fence_init();
     }
+    for (int idx = threadIdx.x; idx < 2 * NW; idx += blockDim.x) bits[idx / NW][idx % NW] = 0u;
     {
         const int npad = NPAD - N;          // H on the left, the rest on the right
         for (int idx = threadIdx.x; idx < 3 * RP * npad; idx += blockDim.x) {
@@ -193,214 +241,73 @@ __global__ void __launch_bounds__(NCC_THREADS, 2) k_detect(const float* __restri
         }
     }
     __syncthreads();
-    // rows [i0-1-H, i0+NCC_RS+1+H) of item `it`'s plane into buffer bb: zero
-    // outside the plane (all threads), one bulk copy inside (thread 0)
-    auto fetch = [&](int it, int bb) {
-        const int plane = it / nstrip, strip = it - plane * nstrip;
-        const int rlo = strip * NCC_RS - 1 - H;
-        const int lo = max(rlo, 0), hi = max(lo, min(rlo + rin, nz));
-        const int z0 = min(lo - rlo, rin), z1 = hi - rlo;
-        float* sA = sm + bb * abuf;
-        for (int idx = threadIdx.x; idx < z0 * N; idx += blockDim.x) sA[idx] = 0.f;
-        for (int idx = threadIdx.x; idx < (rin - z1) * N; idx += blockDim.x) sA[(size_t)z1 * N + idx] = 0.f;
-        if (threadIdx.x == 0) {
+    if (threadIdx.x >= NT) {
+        // ---- serving warp
+        const int lane = threadIdx.x - NT;
+        // rows [i0-1-H, i0+NCC_RS+1+H) of item `it`'s plane into buffer bb: zero
+        // outside the plane, one bulk copy inside
+        auto fetch = [&](int it, int bb) {
+            const int plane = it / nstrip, strip = it - plane * nstrip;
+            const int rlo = strip * NCC_RS - 1 - H;
+            const int lo = max(rlo, 0), hi = max(lo, min(rlo + rin, nz));
+            const int z0 = min(lo - rlo, rin), z1 = hi - rlo;
+            float* sA = sm + bb * abuf;
+            for (int idx = lane; idx < z0 * N; idx += 32) sA[idx] = 0.f;
+            for (int idx = lane; idx < (rin - z1) * N; idx += 32) sA[(size_t)z1 * N + idx] = 0.f;
             fence_proxy_async();
-            // the copied rows land inside the buffer's rin rows (checked build; else nothing is copied)
-            const bool in = chk(lo >= rlo && hi - rlo <= rin && plane < nplanes, status);
-            const unsigned bytes = in ? (unsigned)((hi - lo) * N * sizeof(float)) : 0u;
-            mbar_arrive_expect_tx(&bar[bb], bytes);
-            if (bytes)
-                bulk_g2s(sA + (size_t)(lo - rlo) * N, A + ((size_t)plane * nz + lo) * N, bytes, &bar[bb]);
-        }
-    };
-    // packed Gaussian taps, held for every item
-    uint64_t gz[D], gl[D];
-#pragma unroll
-    for (int q = 0; q < D; ++q) {
-        gz[q] = f2_pack(nc.gz[q], nc.gz[q]);
-        gl[q] = f2_pack(nc.gl[q], nc.gl[q]);
-    }
-    int it = blockIdx.x;
-    if (it < items) fetch(it, 0);
-    for (int k = 0; it < items; it += gridDim.x, ++k) {
-        const int bb = k & 1;
-        const int next = it + gridDim.x;
-        // the other buffer was released by the barrier that ended the previous item
-        if (next < items) fetch(next, bb ^ 1);
-        if (!cta_wait_copies(&bar[bb], (unsigned)(k >> 1) & 1u, status)) {
-            if (next < items) mbar_wait_bounded(&bar[bb ^ 1], (unsigned)((k + 1) >> 1) & 1u);
-            return;
-        }
-        float* sA = sm + bb * abuf;
-        float* sN = sA;                     // NCC rows over the amplitude rows once the vertical pass is done
-        const int plane = it / nstrip, strip = it - plane * nstrip;
-        const int t = plane / (2 * S), axis = (plane / S) % 2, b = plane % S;
-        const int i0 = strip * NCC_RS;
-        const float Mt = Mf[t];
-        const float athr = nc.alpha * Mt;
-        for (int idx = threadIdx.x; idx < NW; idx += blockDim.x) bits[idx] = 0u;
-        // ---- vertical pass: thread = (column pair, VB output rows)
-        {
-            const int NP = N / 2;
-            const unsigned sAa = smem_u32(sA), sVa = smem_u32(sV);
-            for (int task = threadIdx.x; task < NP * (RN / VB); task += blockDim.x) {
-                const int cp = task % NP, rb = task / NP;
-                const int ro0 = rb * VB;
-                // NCC rows ro0 .. ro0 + VB - 1 use amplitude rows ro0 .. ro0 + VB - 1 + 2H
-                uint64_t x[VB + 2 * H];
-                const unsigned src = sAa + (unsigned)((ro0 * N + 2 * cp) * 4);
-#pragma unroll
-                for (int m = 0; m < VB + 2 * H; ++m) x[m] = lds_u64(src + (unsigned)(m * N * 4));
-#pragma unroll
-                for (int r = 0; r < VB; ++r) {
-                    // the centre amplitude of NCC row ro0 + r, both columns of the pair
-                    const float2 ac = f2_unpack(x[r + H]);
-                    const unsigned short fl = (unsigned short)((ac.x >= athr ? 1u : 0u) | (ac.y >= athr ? 0x100u : 0u));
-                    if (chk((ro0 + r) * N + 2 * cp + 1 < RN * N, status))
-                        *reinterpret_cast<unsigned short*>(aflag + (ro0 + r) * N + 2 * cp) = fl;
-                }
-                uint64_t v1[VB], v2[VB], vg[VB];
-                split_box<H, VB>([&](int q) { return x[q]; }, v1);
-                split_box<H, VB>([&](int q) { return f2_mul(x[q], x[q]); }, v2);
-#pragma unroll
-                for (int r = 0; r < VB; ++r) {
-                    uint64_t a = f2_mul(gz[0], x[r]);
-#pragma unroll
-                    for (int q = 1; q < D; ++q) a = f2_fma(gz[q], x[r + q], a);
-                    vg[r] = a;
-                }
-                // transpose 2 x 2 blocks into row pairs: [arr][rp][H + column][row parity]
-                const unsigned dst0 = sVa + (unsigned)(((ro0 / 2) * VS + 2 * (2 * cp + H)) * 4);
-#pragma unroll
-                for (int j = 0; j < VB; j += 2) {
-                    const uint64_t* arrs[3] = {v1, v2, vg};
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        const float2 r0 = f2_unpack(arrs[a][j]), r1 = f2_unpack(arrs[a][j + 1]);
-                        const unsigned dst = dst0 + (unsigned)(((a * RP + j / 2) * VS) * 4);
-                        asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(r0.x), "f"(r1.x) : "memory");
-                        asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(dst + 8u), "f"(r0.y), "f"(r1.y) : "memory");
-                    }
-                }
+            __syncwarp();
+            if (lane == 0) {
+                // the copied rows land inside the buffer's rin rows (checked build; else nothing is copied)
+                const bool in = chk(lo >= rlo && hi - rlo <= rin && plane < nplanes, status);
+                const unsigned bytes = in ? (unsigned)((hi - lo) * N * sizeof(float)) : 0u;
+                mbar_arrive_expect_tx(&full[bb], bytes);
+                if (bytes)
+                    bulk_g2s(sA + (size_t)(lo - rlo) * N, A + ((size_t)plane * nz + lo) * N, bytes, &full[bb]);
             }
-        }
-        __syncthreads();
-        // ---- horizontal pass + NCC: thread = (row pair, HB output columns);
-        // the amplitude rows are no longer read, so the NCC rows take their place
-        {
-            const float flat = nc.flat_coef * Mt * Mt;
-            const float inv_d2 = 1.0f / (float)(D * D);
-            const int ncb = (N + HB - 1) / HB;
-            const uint64_t nid2 = f2_pack(-inv_d2, -inv_d2), nmu = f2_pack(-nc.muG, -nc.muG);
-            const unsigned sVa = smem_u32(sV);
-            for (int task = threadIdx.x; task < RP * ncb; task += blockDim.x) {
-                const int rp = task % RP, cb = task / RP;
-                const int c0 = cb * HB;
-                // padded input columns c0 - H .. c0 + HB - 1 + H start at pad index c0; past N they
-                // read the right pad (zero) or feed only outputs past N
-                const unsigned at = sVa + (unsigned)((rp * VS + 2 * c0) * 4);
-                uint64_t s1[HB], s2[HB], sg[HB];
-                {
-                    uint64_t a[HB + 2 * H];
-#pragma unroll
-                    for (int m = 0; m < HB + 2 * H; ++m) a[m] = lds_u64(at + (unsigned)(m * 8));
-                    split_box<H, HB>([&](int q) { return a[q]; }, s1);
-#pragma unroll
-                    for (int m = 0; m < HB + 2 * H; ++m) a[m] = lds_u64(at + (unsigned)(RP * VS * 4 + m * 8));
-                    split_box<H, HB>([&](int q) { return a[q]; }, s2);
-#pragma unroll
-                    for (int m = 0; m < HB + 2 * H; ++m) a[m] = lds_u64(at + (unsigned)(2 * RP * VS * 4 + m * 8));
-#pragma unroll
-                    for (int r = 0; r < HB; ++r) {
-                        uint64_t g = f2_mul(gl[0], a[r]);
-#pragma unroll
-                        for (int q = 1; q < D; ++q) g = f2_fma(gl[q], a[r + q], g);
-                        sg[r] = g;
-                    }
-                }
-                const int ia = i0 - 1 + 2 * rp;    // plane row of the pair's first row
-                const bool row0 = ia >= H && ia < nz - H && Mt > 0.f;
-                const bool row1 = ia + 1 >= H && ia + 1 < nz - H && Mt > 0.f;
-                float* nrow = sN + (2 * rp) * NS + c0;
-#pragma unroll
-                for (int j = 0; j < HB; ++j) {
-                    const int c = c0 + j;
-                    if (c >= N) break;
-                    // ssA = s2 - s1^2 / d^2, numerator = sg - mu_G s1 (both rows of the pair)
-                    const float2 ss = f2_unpack(f2_fma(f2_mul(s1[j], s1[j]), nid2, s2[j]));
-                    const float2 nu = f2_unpack(f2_fma(nmu, s1[j], sg[j]));
-                    const bool colok = c >= H && c < N - H;
-                    const float v0 = (colok && row0 && ss.x > flat) ? nu.x * nc.inv_ssG_sqrt * rsqrtf(ss.x) : 0.f;
-                    const float v1 = (colok && row1 && ss.y > flat) ? nu.y * nc.inv_ssG_sqrt * rsqrtf(ss.y) : 0.f;
-                    nrow[j] = v0;
-                    nrow[NS + j] = v1;
-                    if (ncc_out) {
-                        if (2 * rp >= 1 && 2 * rp <= NCC_RS && ia < nz) ncc_out[((size_t)plane * nz + ia) * N + c] = v0;
-                        if (2 * rp + 1 <= NCC_RS && ia + 1 < nz) ncc_out[((size_t)plane * nz + ia + 1) * N + c] = v1;
-                    }
-                }
+            __syncwarp();
+        };
+        const int stride = gridDim.x;
+        int fetched = 0;                    // items fetched so far
+        for (int it = blockIdx.x; it < items && fetched < 2; it += stride, ++fetched) fetch(it, fetched);
+        int k = 0;
+        for (int it = blockIdx.x; it < items; it += stride, ++k) {
+            const int bb = k & 1;
+            if (!mbar_wait_bounded(&done[bb], (unsigned)(k >> 1) & 1u)) {
+                if (lane == 0) atomicOr(status, ST_TIMEOUT);
+                break;
             }
-        }
-        __syncthreads();
-        // ---- peaks: test every strip pixel (thread = column, rows in steps), mark
-        // the candidates in a raster-order bitmap, then compact the bitmap words
-        // (consecutive words per thread, a block-wide exclusive scan of their
-        // counts) so the strip's candidates come out in raster order
-        {
-            const int RG = NCC_THREADS / N > 0 ? NCC_THREADS / N : 1;   // row groups (N <= 256)
-            const int l = threadIdx.x % N, rg = threadIdx.x / N;
-            // NCC rows whose plane row i = i0 - 1 + ro lies in [1, nz - 2]
-            const int ro_lo = max(1, 2 - i0), ro_hi = min(NCC_RS, nz - 1 - i0);
-            if (rg < RG && l >= 1 && l < N - 1) {
-                int ro = ro_lo + rg;
-                const float* np_ = sN + ro * NS + l;
-#pragma unroll 5
-                for (; ro <= ro_hi; ro += RG, np_ += RG * NS) {
-                    const float c = *np_;
-                    if (!(c >= nc.ncc_min)) continue;
-                    bool pk = aflag[ro * N + l] != 0;
-#pragma unroll
-                    for (int a = -1; a <= 1; ++a)
-#pragma unroll
-                        for (int bq = -1; bq <= 1; ++bq) {
-                            if (a == 0 && bq == 0) continue;
-                            const float q = sN[(ro + a) * NS + l + bq];
-                            const bool earlier = (a < 0) || (a == 0 && bq < 0);
-                            pk = pk && (earlier ? (c > q) : (c >= q));
-                        }
-                    if (pk) {
-                        const int p = (ro - 1) * N + l;
-                        if (chk(p >= 0 && (p >> 5) < NW && ro + 1 < RN, status)) atomicOr(&bits[p >> 5], 1u << (p & 31));
-                    }
+            const float* sN = sm + bb * abuf;
+            const int plane = it / nstrip, strip = it - plane * nstrip;
+            const int t = plane / (2 * S), axis = (plane / S) % 2, b = plane % S, i0 = strip * NCC_RS;
+            const int n_over = nlist[bb];
+            if (n_over <= DET_LIST)
+                for (int q = lane; q < n_over; q += 32) {
+                    const int p = list[bb][q], ro = 1 + p / N;
+                    if (ncc_peak(sN, NS, ro, p - (ro - 1) * N) && chk((p >> 5) < NW && ro + 1 < RN, status))
+                        atomicOr(&bits[bb][p >> 5], 1u << (p & 31));
                 }
+            __syncwarp();
+            // lane: a run of bitmap words; their counts scanned over the warp
+            const int wpl = (nwords + 31) / 32, w0 = lane * wpl, w1 = min(nwords, w0 + wpl);
+            int x = 0;
+            for (int w = w0; w < w1; ++w) x += __popc(bits[bb][w]);
+            int before = -x;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
             }
-        }
-        __syncthreads();
-        ulm_loc2d* slot = cand + (size_t)it * CAND_CAP;
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        // each thread compacts wpt consecutive bitmap words (wpt = 2 only when N > 273)
-        const int nwords = (NCC_RS * N + 31) / 32;
-        const int wpt = (nwords + NCC_THREADS - 1) / NCC_THREADS;
-        const int w0 = threadIdx.x * wpt;
-        unsigned long long mask = 0ull;
-        if (w0 < nwords) mask = bits[w0];
-        if (wpt == 2 && w0 + 1 < nwords) mask |= (unsigned long long)bits[w0 + 1] << 32;
-        const int mine = __popcll(mask);
-        int x = mine;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) wsum[warp] = x;
-        __syncthreads();
-        int before = x - mine;
-        for (int w = 0; w < warp; ++w) before += wsum[w];
-        while (mask) {
-            const int bit = __ffsll(mask) - 1;
-            mask &= mask - 1;
-            if (before < CAND_CAP) {
-                const int p = w0 * 32 + bit;
-                const int ro = 1 + p / N, l = p - (ro - 1) * N, i = i0 - 1 + ro;
+            before += x;
+            if (lane == 31) slot_count(cnt, part, total, it, x, status);
+            for (int w = w0; w < w1; ++w) {
+                unsigned m = bits[bb][w];
+                bits[bb][w] = 0u;
+                for (; m; m &= m - 1, ++before)
+                    if (before < CAND_CAP) order[before] = (unsigned short)(w * 32 + __ffs(m) - 1);
+            }
+            __syncwarp();
+            const int npk = min(__shfl_sync(0xffffffffu, x, 31), CAND_CAP);
+            for (int q = lane; q < npk; q += 32) {
+                const int p = order[q], ro = 1 + p / N, l = p - (ro - 1) * N, i = i0 - 1 + ro;
                 const float c = sN[ro * NS + l];
                 auto para = [](float fm, float f0, float fp) {
                     const float den = fm - 2.f * f0 + fp;
@@ -417,24 +324,202 @@ __global__ void __launch_bounds__(NCC_THREADS, 2) k_detect(const float* __restri
                 e.z = (float)i + para(sN[(ro - 1) * NS + l], c, sN[(ro + 1) * NS + l]);
                 e.lat = (float)l + para(sN[ro * NS + l - 1], c, sN[ro * NS + l + 1]);
                 e.ncc = c;
-                e.amp = 0.f;        // filled from A by the gather (no global load in this phase)
+                e.amp = 0.f;        // filled from A by the gather
                 e.reserved = 0;
-                slot[before] = e;
+                cand[(size_t)it * CAND_CAP + q] = e;
             }
-            ++before;
+            if (lane == 0) nlist[bb] = 0;
+            __syncwarp();
+            // the buffer, its list and its bitmap are free: the item after the next
+            if (it + 2 * stride < items) {
+                fetch(it + 2 * stride, bb);
+                ++fetched;
+            }
         }
-        // the last thread's running index is the strip's count
-        if (threadIdx.x == blockDim.x - 1) {
-            cnt[it] = before;
-            if (before > CAND_CAP) atomicOr(status, ST_CAPACITY);
+        // a wait ran out: the copies in flight end (bounded) before the block may
+        for (int q = k; q < fetched; ++q) mbar_wait_bounded(&full[q & 1], (unsigned)(q >> 1) & 1u);
+    } else {
+        // packed Gaussian taps, held for every item
+        uint64_t gz[D], gl[D];
+#pragma unroll
+        for (int q = 0; q < D; ++q) {
+            gz[q] = f2_pack(nc.gz[q], nc.gz[q]);
+            gl[q] = f2_pack(nc.gl[q], nc.gl[q]);
         }
-        // the next iteration fetches into this buffer and rewrites the bitmap
-        __syncthreads();
+        int k = 0;
+        // strip, plane of its frame and frame of the item, advanced without divisions
+        const int dstrip = gridDim.x % nstrip, dpl = gridDim.x / nstrip % (2 * S), dt = gridDim.x / nstrip / (2 * S);
+        int strip = blockIdx.x % nstrip, pl = blockIdx.x / nstrip % (2 * S), t = blockIdx.x / nstrip / (2 * S);
+        float Mnext = blockIdx.x < items ? __ldg(Mf + t) : 0.f;
+        for (int it = blockIdx.x; it < items; it += gridDim.x, ++k) {
+            const int bb = k & 1;
+            const float Mt = Mnext;
+            const int plane = t * 2 * S + pl, i0 = strip * NCC_RS;
+            strip += dstrip, pl += dpl, t += dt;
+            if (strip >= nstrip) strip -= nstrip, ++pl;
+            if (pl >= 2 * S) pl -= 2 * S, ++t;
+            if (it + (int)gridDim.x < items) Mnext = __ldg(Mf + t);
+            const int late = !mbar_wait_bounded(&full[bb], (unsigned)(k >> 1) & 1u);
+            float* sA = sm + bb * abuf;
+            float* sN = sA;                     // NCC rows over the amplitude rows once the vertical pass is done
+            const float athr = nc.alpha * Mt;
+            // NCC rows whose plane row i = i0 - 1 + ro lies in [1, nz - 2]
+            const int ro_lo = max(1, 2 - i0), ro_hi = min(NCC_RS, nz - 1 - i0);
+            // ---- vertical pass: thread = (column pair, VB output rows)
+            {
+                const int NP = N / 2;
+                const unsigned sAa = smem_u32(sA), sVa = smem_u32(sV);
+                for (int task = threadIdx.x; task < NP * (RN / VB); task += NT) {
+                    const int cp = task % NP, rb = task / NP;
+                    const int ro0 = rb * VB;
+                    // NCC rows ro0 .. ro0 + VB - 1 use amplitude rows ro0 .. ro0 + VB - 1 + 2H
+                    uint64_t x[VB + 2 * H];
+                    const unsigned src = sAa + (unsigned)((ro0 * N + 2 * cp) * 4);
+#pragma unroll
+                    for (int m = 0; m < VB + 2 * H; ++m) x[m] = lds_u64(src + (unsigned)(m * N * 4));
+#pragma unroll
+                    for (int r = 0; r < VB; ++r) {
+                        // the centre amplitude of NCC row ro0 + r, both columns of the pair
+                        const float2 ac = f2_unpack(x[r + H]);
+                        const unsigned short fl = (unsigned short)((ac.x >= athr ? 1u : 0u) | (ac.y >= athr ? 0x100u : 0u));
+                        if (chk((ro0 + r) * N + 2 * cp + 1 < RN * N, status))
+                            *reinterpret_cast<unsigned short*>(aflag + (ro0 + r) * N + 2 * cp) = fl;
+                    }
+                    uint64_t v1[VB], v2[VB], vg[VB];
+                    split_box<H, VB>([&](int q) { return x[q]; }, v1);
+                    split_box<H, VB>([&](int q) { return f2_mul(x[q], x[q]); }, v2);
+#pragma unroll
+                    for (int r = 0; r < VB; ++r) {
+                        uint64_t a = f2_mul(gz[0], x[r]);
+#pragma unroll
+                        for (int q = 1; q < D; ++q) a = f2_fma(gz[q], x[r + q], a);
+                        vg[r] = a;
+                    }
+                    // transpose 2 x 2 blocks into row pairs: [arr][rp][H + column][row parity]
+                    const unsigned dst0 = sVa + (unsigned)(((ro0 / 2) * VS + 2 * (2 * cp + H)) * 4);
+#pragma unroll
+                    for (int j = 0; j < VB; j += 2) {
+                        const uint64_t* arrs[3] = {v1, v2, vg};
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+                            const float2 r0 = f2_unpack(arrs[a][j]), r1 = f2_unpack(arrs[a][j + 1]);
+                            const unsigned dst = dst0 + (unsigned)(((a * RP + j / 2) * VS) * 4);
+                            asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(r0.x), "f"(r1.x) : "memory");
+                            asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(dst + 8u), "f"(r0.y), "f"(r1.y) : "memory");
+                        }
+                    }
+                }
+            }
+            // the vertical sums are complete; every thread's wait for the rows succeeded
+            int any;
+            asm volatile(
+                "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 q, %1, 0;\n\tbarrier.cta.red.or.pred p, 1, %2, q;\n\tselp.s32 %0, 1, 0, p;\n\t}"
+                : "=r"(any)
+                : "r"(late), "n"(NT)
+                : "memory");
+            if (any) {
+                if (threadIdx.x == 0) atomicOr(status, ST_TIMEOUT);
+                break;
+            }
+            // ---- horizontal pass + NCC: thread = (row pair, HB output columns);
+            // the amplitude rows are no longer read, so the NCC rows take their place
+            {
+                const float flat = nc.flat_coef * Mt * Mt;
+                const float inv_d2 = 1.0f / (float)(D * D);
+                const int ncb = (N + HB - 1) / HB;
+                const uint64_t nid2 = f2_pack(-inv_d2, -inv_d2), nmu = f2_pack(-nc.muG, -nc.muG);
+                const unsigned sVa = smem_u32(sV);
+                for (int task = threadIdx.x; task < RP * ncb; task += NT) {
+                    const int rp = task % RP, cb = task / RP;
+                    const int c0 = cb * HB;
+                    // padded input columns c0 - H .. c0 + HB - 1 + H start at pad index c0; past N they
+                    // read the right pad (zero) or feed only outputs past N
+                    const unsigned at = sVa + (unsigned)((rp * VS + 2 * c0) * 4);
+                    uint64_t s1[HB], s2[HB], sg[HB];
+                    {
+                        uint64_t a[HB + 2 * H];
+#pragma unroll
+                        for (int m = 0; m < HB + 2 * H; ++m) a[m] = lds_u64(at + (unsigned)(m * 8));
+                        split_box<H, HB>([&](int q) { return a[q]; }, s1);
+#pragma unroll
+                        for (int m = 0; m < HB + 2 * H; ++m) a[m] = lds_u64(at + (unsigned)(RP * VS * 4 + m * 8));
+                        split_box<H, HB>([&](int q) { return a[q]; }, s2);
+#pragma unroll
+                        for (int m = 0; m < HB + 2 * H; ++m) a[m] = lds_u64(at + (unsigned)(2 * RP * VS * 4 + m * 8));
+#pragma unroll
+                        for (int r = 0; r < HB; ++r) {
+                            uint64_t g = f2_mul(gl[0], a[r]);
+#pragma unroll
+                            for (int q = 1; q < D; ++q) g = f2_fma(gl[q], a[r + q], g);
+                            sg[r] = g;
+                        }
+                    }
+                    const int ia = i0 - 1 + 2 * rp;    // plane row of the pair's first row
+                    const bool row0 = ia >= H && ia < nz - H && Mt > 0.f;
+                    const bool row1 = ia + 1 >= H && ia + 1 < nz - H && Mt > 0.f;
+                    float* nrow = sN + (2 * rp) * NS + c0;
+                    unsigned over = 0u;                // pixels with NCC >= ncc_min: bits j (first row) and HB + j
+#pragma unroll
+                    for (int j = 0; j < HB; ++j) {
+                        const int c = c0 + j;
+                        if (c >= N) break;
+                        // ssA = s2 - s1^2 / d^2, numerator = sg - mu_G s1 (both rows of the pair)
+                        const float2 ss = f2_unpack(f2_fma(f2_mul(s1[j], s1[j]), nid2, s2[j]));
+                        const float2 nu = f2_unpack(f2_fma(nmu, s1[j], sg[j]));
+                        const bool colok = c >= H && c < N - H;
+                        const float v0 = (colok && row0 && ss.x > flat) ? nu.x * nc.inv_ssG_sqrt * rsqrtf(ss.x) : 0.f;
+                        const float v1 = (colok && row1 && ss.y > flat) ? nu.y * nc.inv_ssG_sqrt * rsqrtf(ss.y) : 0.f;
+                        nrow[j] = v0;
+                        nrow[NS + j] = v1;
+                        if (v0 >= nc.ncc_min) over |= 1u << j;
+                        if (v1 >= nc.ncc_min) over |= 1u << (HB + j);
+                        if (ncc_out) {
+                            if (2 * rp >= 1 && 2 * rp <= NCC_RS && ia < nz) ncc_out[((size_t)plane * nz + ia) * N + c] = v0;
+                            if (2 * rp + 1 <= NCC_RS && ia + 1 < nz) ncc_out[((size_t)plane * nz + ia + 1) * N + c] = v1;
+                        }
+                    }
+                    // the rows and columns a peak may lie in
+                    constexpr unsigned RM = (1u << HB) - 1u;
+                    if (2 * rp < ro_lo || 2 * rp > ro_hi) over &= ~RM;
+                    if (2 * rp + 1 < ro_lo || 2 * rp + 1 > ro_hi) over &= RM;
+                    if (c0 == 0) over &= ~(1u | 1u << HB);
+                    if (c0 + HB >= N) over &= ~(1u << (N - 1 - c0) | 1u << (HB + N - 1 - c0));
+                    while (over) {
+                        const int bit = __ffs(over) - 1;
+                        over &= over - 1;
+                        const int ro = 2 * rp + (bit >= HB), l = c0 + (bit >= HB ? bit - HB : bit);
+                        if (!aflag[ro * N + l]) continue;
+                        const int at = atomicAdd(&nlist[bb], 1);
+                        if (at < DET_LIST) list[bb][at] = (unsigned short)((ro - 1) * N + l);
+                    }
+                }
+            }
+            asm volatile("barrier.cta.sync 1, %0;" ::"n"(NT) : "memory");
+            if (nlist[bb] > DET_LIST) {
+                // many pixels over the thresholds: every thread tests the strip's pixels
+                constexpr int MAXL = NT;
+                const int RG = MAXL / N > 0 ? MAXL / N : 1;
+                for (int l = threadIdx.x % min(N, MAXL); l < N; l += MAXL)
+                    for (int ro = ro_lo + (N < MAXL ? threadIdx.x / N : 0); ro <= ro_hi; ro += RG)
+                        if ((N >= MAXL || threadIdx.x / N < RG) && l >= 1 && l < N - 1 && sN[ro * NS + l] >= nc.ncc_min &&
+                            aflag[ro * N + l] && ncc_peak(sN, NS, ro, l)) {
+                            const int p = (ro - 1) * N + l;
+                            if (chk(p >= 0 && (p >> 5) < NW && ro + 1 < RN, status)) atomicOr(&bits[bb][p >> 5], 1u << (p & 31));
+                        }
+                // the flags are overwritten by the next item's vertical pass
+                asm volatile("barrier.cta.sync 1, %0;" ::"n"(NT) : "memory");
+            }
+            __syncwarp();
+            if ((threadIdx.x & 31) == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&done[bb])) : "memory");
+        }
     }
-    if (threadIdx.x == 0) {
-        mbar_inval(&bar[0]);
-        mbar_inval(&bar[1]);
-    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int q = 0; q < 2; ++q) {
+            mbar_inval(&full[q]);
+            mbar_inval(&done[q]);
+        }
 }
 
 // ---------------------------------------------------------------------------
@@ -445,6 +530,7 @@ __global__ void __launch_bounds__(NCC_THREADS, 2) k_detect(const float* __restri
 __global__ void __launch_bounds__(256) k_detect_map(const float* __restrict__ map, int up, const float* __restrict__ A,
                                                     const float* __restrict__ Mf, int S, int nz, int N, float score_min,
                                                     float alpha, ulm_loc2d* __restrict__ cand, int* __restrict__ cnt,
+                                                    int* __restrict__ part, unsigned long long* __restrict__ total,
                                                     unsigned* __restrict__ status)
 {
     extern __shared__ __align__(128) float smf[];
@@ -557,145 +643,81 @@ __global__ void __launch_bounds__(256) k_detect_map(const float* __restrict__ ma
         }
     }
     // the last thread's running index is the strip's count
-    if (threadIdx.x == blockDim.x - 1) {
-        cnt[(size_t)plane * nstrip + strip] = before;
-        if (before > CAND_CAP) atomicOr(status, ST_CAPACITY);
-    }
+    if (threadIdx.x == blockDim.x - 1) slot_count(cnt, part, total, plane * nstrip + strip, before, status);
 }
 
-// Multi-block exclusive scan of min(cnt[i], cap_each) (cap_each <= 0: no cap)
-// over n entries (n = min(n, *n_dev) when n_dev is given).  off[n] = kept
-// total; *total_true = sum of the uncapped counts.
-#define SCAN_CHUNK 4096
-#define SCAN_THREADS 512
+#define SCAN_MAX (1024 * 4096)   // entries of one compaction at most
 
-__device__ __forceinline__ int scan_n(int n, const int* n_dev) { return n_dev ? min(n, *n_dev) : n; }
-
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_part(const int* __restrict__ cnt, int n, const int* __restrict__ n_dev,
-                                                            int cap_each, long long* __restrict__ part)
+// sum over the block of part[0 .. n) plus `own` of every thread before this one:
+// the exclusive offset of this thread's first entry; *all: the sum with every
+// thread's own (256 threads)
+__device__ __forceinline__ int block_offset(const int* __restrict__ part, int n, int own, int* red, int* all)
 {
-    __shared__ long long red[2][SCAN_THREADS / 32];
-    n = scan_n(n, n_dev);
-    const int lo = blockIdx.x * SCAN_CHUNK, hi = min(n, lo + SCAN_CHUNK);
-    long long s = 0, st = 0;
-    for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        const int c = cnt[i];
-        st += c;
-        s += (cap_each > 0) ? min(c, cap_each) : c;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        s += __shfl_xor_sync(0xffffffffu, s, o);
-        st += __shfl_xor_sync(0xffffffffu, st, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        red[0][threadIdx.x >> 5] = s;
-        red[1][threadIdx.x >> 5] = st;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        long long a = 0, b = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            a += red[0][w];
-            b += red[1][w];
-        }
-        part[2 * blockIdx.x] = a;
-        part[2 * blockIdx.x + 1] = b;
-    }
-}
-
-// one block: exclusive scan of the per-chunk totals (nb <= 1024 chunks)
-__global__ void __launch_bounds__(1024) k_scan_top(long long* __restrict__ part, int nb, int n,
-                                                   const int* __restrict__ n_dev, int* __restrict__ off,
-                                                   int* __restrict__ total_true)
-{
-    __shared__ long long a[1024], b[1024];
-    n = scan_n(n, n_dev);
-    const int used = (n + SCAN_CHUNK - 1) / SCAN_CHUNK;
-    const int i = threadIdx.x;
-    a[i] = (i < nb && i < used) ? part[2 * i] : 0;
-    b[i] = (i < nb && i < used) ? part[2 * i + 1] : 0;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-        long long va = i >= o ? a[i - o] : 0, vb = i >= o ? b[i - o] : 0;
-        __syncthreads();
-        a[i] += va;
-        b[i] += vb;
-        __syncthreads();
-    }
-    if (i < nb) part[2 * i] = i ? a[i - 1] : 0;  // exclusive chunk offset
-    if (i == 1023) {
-        off[n] = (int)min(a[1023], (long long)0x7fffffff);
-        if (total_true) *total_true = (int)min(b[1023], (long long)0x7fffffff);
-    }
-}
-
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(const int* __restrict__ cnt, int n,
-                                                             const int* __restrict__ n_dev, int cap_each,
-                                                             const long long* __restrict__ part, int* __restrict__ off)
-{
-    constexpr int PER = SCAN_CHUNK / SCAN_THREADS;
-    __shared__ int wsum[SCAN_THREADS / 32];
-    n = scan_n(n, n_dev);
-    const int lo = blockIdx.x * SCAN_CHUNK;
-    if (lo >= n) return;
-    const int base = lo + threadIdx.x * PER;
-    int v[PER], s = 0;
-#pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        const int i = base + q;
-        const int c = i < n ? cnt[i] : 0;
-        v[q] = (cap_each > 0) ? min(c, cap_each) : c;
-        s += v[q];
-    }
-    // block exclusive scan of the per-thread sums
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int x = s;
+    int p = 0, x = own;
+    for (int q = threadIdx.x; q < n; q += blockDim.x) p += part[q];
+    p = __reduce_add_sync(0xffffffffu, p);
     for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
     }
-    if (lane == 31) wsum[warp] = x;
+    __syncthreads();                                   // red is free
+    if (lane == 31) red[warp] = x, red[8 + warp] = p;
     __syncthreads();
-    int wpre = 0;
-    for (int w = 0; w < warp; ++w) wpre += wsum[w];
-    int run = (int)part[2 * blockIdx.x] + wpre + x - s;
+    int before = 0, sum = 0;
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        const int i = base + q;
-        if (i < n) off[i] = run;
-        run += v[q];
+    for (int w = 0; w < 8; ++w) {
+        before += red[8 + w];
+        sum += red[w] + red[8 + w];
+        if (w < warp) before += red[w];
     }
+    *all = sum;
+    return before + x - own;
 }
 
-// Copy each strip's kept candidates to their place in the output list.
-// A non-null: each entry's amplitude is read here from A [plane][nz][N] at its
-// pixel (the detection kernel leaves it to this highly parallel pass)
-__global__ void k_gather(const ulm_loc2d* __restrict__ cand, const int* __restrict__ cnt, const int* __restrict__ off,
-                         int nslots, ulm_loc2d* __restrict__ out, int cap, const float* __restrict__ A, int S, int nz,
-                         int N, unsigned* __restrict__ status)
+// Copy the kept candidates of a chunk of slots to their place in the output list:
+// the chunk's offset is the sum of the totals before it, a slot's a scan of the
+// counts in the block (one launch instead of three scan kernels and a gather), and
+// the chunk's entries are spread over its threads.  A non-null: each entry's
+// amplitude is read here from A [plane][nz][N] at its pixel (the detection kernel
+// leaves it to this highly parallel pass).  poff (optional): the list offset of
+// every plane, of nstrip slots each.
+__global__ void __launch_bounds__(256) k_gather(const ulm_loc2d* __restrict__ cand, const int* __restrict__ cnt,
+                                                const int* __restrict__ part, const unsigned long long* __restrict__ total,
+                                                int nslots, int nstrip, ulm_loc2d* __restrict__ out, int cap,
+                                                int* __restrict__ n_out, int* __restrict__ poff, const float* __restrict__ A,
+                                                int S, int nz, int N, unsigned* __restrict__ status)
 {
-    const int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (s >= nslots) return;
-    const int lane = threadIdx.x & 31;
-    const int c = min(cnt[s], CAND_CAP);
-    for (int r = lane; r < c; r += 32) {
-        int dst = off[s] + r;
-        if (dst < cap) {
-            ulm_loc2d e = cand[(size_t)s * CAND_CAP + r];
-            if (A && chk(e.iz >= 0 && e.iz < nz && e.ilat >= 0 && e.ilat < N && e.slab >= 0 && e.slab < S, status))
-                e.amp = __ldg(A + (((size_t)(e.frame * 2 + e.axis) * S + e.slab) * nz + e.iz) * N + e.ilat);
-            out[dst] = e;
-        } else {
+    static_assert(GATHER_SLOTS == 256, "a thread per slot");
+    __shared__ int red[16], off[GATHER_SLOTS + 1];
+    const int s0 = blockIdx.x * GATHER_SLOTS, s = s0 + threadIdx.x;
+    const int own = s < nslots ? min(cnt[s], CAND_CAP) : 0;
+    int all;
+    const int at = block_offset(part, blockIdx.x, own, red, &all);
+    off[threadIdx.x] = at;
+    if (threadIdx.x == 0) off[GATHER_SLOTS] = all;
+    if (poff) {
+        if (s < nslots && s % nstrip == 0) poff[s / nstrip] = at;
+        if (s == nslots - 1) poff[nslots / nstrip] = at + own;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) *n_out = (int)min(*total, 0x7fffffffull);
+    __syncthreads();
+    const int base = off[0], n = all - base;
+    for (int i = threadIdx.x; i < n; i += 256) {
+        const int dst = base + i;
+        if (dst >= cap) {
             atomicOr(status, ST_CAPACITY);
+            break;
         }
+        int lo = 0;                                    // the last slot with off <= dst
+#pragma unroll
+        for (int h = GATHER_SLOTS / 2; h > 0; h >>= 1)
+            if (off[lo + h] <= dst) lo += h;
+        ulm_loc2d e = cand[(size_t)(s0 + lo) * CAND_CAP + (dst - off[lo])];
+        if (A && chk(e.iz >= 0 && e.iz < nz && e.ilat >= 0 && e.ilat < N && e.slab >= 0 && e.slab < S, status))
+            e.amp = __ldg(A + (((size_t)(e.frame * 2 + e.axis) * S + e.slab) * nz + e.iz) * N + e.ilat);
+        out[dst] = e;
     }
-}
-
-// plane offsets of the (frame, axis, slab)-sorted list: first entry of each plane
-__global__ void k_strip_to_plane(const int* __restrict__ off, int nstrip, int nplanes, int* __restrict__ poff)
-{
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p <= nplanes) poff[p] = off[(size_t)p * nstrip];
 }
 
 // ---------------------------------------------------------------------------
@@ -727,7 +749,7 @@ __global__ void k_list_plane_offsets(const ulm_loc2d* __restrict__ L, const int*
 // fl32(e) > 1 implies e > 1 and fl32(e) < 1 implies e < 1; a ratio more than
 // 0.01 inside or outside a bound is on the same side in FP64), and in FP64
 // only when the FP32 value sits at the bound.
-__device__ __forceinline__ bool pair_ok(const ulm_loc2d& x, const ulm_loc2d& y, int P, double* cost)
+__device__ __forceinline__ bool pair_ok(const ulm_loc2d& x, const ulm_loc2d& y, int P)
 {
     if (x.frame != y.frame) return false;
     // x.ilat / P == y.slab and y.ilat / P == x.slab (non-negative indexes), without divisions
@@ -744,96 +766,197 @@ __device__ __forceinline__ bool pair_ok(const ulm_loc2d& x, const ulm_loc2d& y, 
         const double r = ax / ay;
         if (!(r >= 0.9 && r <= 1.11)) return false;
     }
-    *cost = ax > ay ? ax / ay : ay / ax;
     return true;
 }
 
-__global__ void k_pair_match(const ulm_loc2d* __restrict__ L, const int* __restrict__ n2d, int cap2d, int S, int P,
-                             const int* __restrict__ poff, int* __restrict__ match)
+// whether partner p (amplitude pa) of an entry of amplitude a beats partner q (qa):
+// the lower FP64 cost max / min, ties to the lower index.  The FP32 costs (1 to 1.12,
+// within 1.4e-7 of the quotient) decide unless they are closer than 4e-7.
+__device__ __forceinline__ bool pair_better(float a, int p, float pa, int q, float qa)
 {
-    const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    const int n = min(*n2d, cap2d);
-    if (a >= n) return;
-    const ulm_loc2d x = L[a];
-    int m = -1;
-    if (x.axis == 0) {
-        const int py = (x.frame * 2 + 1) * S + x.ilat / P;
-        int best = -1;
-        double bc = 0.0;
-        for (int q = poff[py]; q < min(poff[py + 1], n); ++q) {
-            double c;
-            if (pair_ok(x, L[q], P, &c) && (best < 0 || c < bc)) {
-                best = q;
-                bc = c;
-            }
-        }
-        if (best >= 0) {
-            const ulm_loc2d y = L[best];
-            const int px = (y.frame * 2 + 0) * S + y.ilat / P;
-            int back = -1;
-            double bc2 = 0.0;
-            for (int q = poff[px]; q < min(poff[px + 1], n); ++q) {
-                double c;
-                if (pair_ok(L[q], y, P, &c) && (back < 0 || c < bc2)) {
-                    back = q;
-                    bc2 = c;
+    const float c = a > pa ? a / pa : pa / a, d = a > qa ? a / qa : qa / a;
+    if (c < d - 4e-7f) return true;
+    if (c > d + 4e-7f) return false;
+    const double A = a, C = pa, D = qa;
+    const double c64 = A > C ? A / C : C / A, d64 = A > D ? A / D : D / A;
+    return c64 < d64 || (c64 == d64 && p < q);
+}
+
+// Every entry's partner on the other axis: the eligible entry of the least cost in
+// the plane of its own slab's counterpart, ties to the lower index (-1: none).  A
+// pair is a match when each is the other's partner.  Eight lanes share an entry (a
+// plane holds a few to a few tens of entries; one thread per XZ entry that searched
+// there and back took 222 us on the paper's list and 25 us on a tiny one, a serial
+// chain of loads and FP64 divisions; now 70 and 5).
+#define PAIR_LANES 8
+__global__ void __launch_bounds__(256) k_pair_best(const ulm_loc2d* __restrict__ L, const int* __restrict__ n2d, int cap2d,
+                                                   int F, int S, int P, const int* __restrict__ poff, int* __restrict__ best)
+{
+    const int n = min(*n2d, cap2d), sub = threadIdx.x % PAIR_LANES;
+    constexpr int PER = 256 / PAIR_LANES;
+    for (int a0 = blockIdx.x * PER; a0 < n; a0 += gridDim.x * PER) {
+        const int a = a0 + threadIdx.x / PAIR_LANES;
+        int b = 0x7fffffff;
+        float amp = 0.f, pa = 0.f;
+        if (a < n) {
+            const ulm_loc2d x = L[a];
+            amp = x.amp;
+            const int slab = x.ilat / P;
+            if ((unsigned)x.axis < 2u && x.frame >= 0 && x.frame < F && x.ilat >= 0 && slab < S) {
+                const int pl = (x.frame * 2 + 1 - x.axis) * S + slab;
+                const int q1 = min(poff[pl + 1], n);
+                for (int q = poff[pl] + sub; q < q1; q += PAIR_LANES) {
+                    const ulm_loc2d y = L[q];
+                    if ((x.axis == 0 ? pair_ok(x, y, P) : pair_ok(y, x, P)) &&
+                        (b == 0x7fffffff || pair_better(amp, q, y.amp, b, pa))) {
+                        b = q;
+                        pa = y.amp;
+                    }
                 }
             }
-            if (back == a) m = best;
+        }
+#pragma unroll
+        for (int o = PAIR_LANES / 2; o > 0; o >>= 1) {
+            const int ob = __shfl_xor_sync(0xffffffffu, b, o);
+            const float oa = __shfl_xor_sync(0xffffffffu, pa, o);
+            if (ob != 0x7fffffff && (b == 0x7fffffff || pair_better(amp, ob, oa, b, pa))) {
+                b = ob;
+                pa = oa;
+            }
+        }
+        if (a < n && sub == 0) best[a] = b == 0x7fffffff ? -1 : b;
+    }
+}
+
+// entry a is the XZ half of a match
+__device__ __forceinline__ bool pair_mutual(const ulm_loc2d* __restrict__ L, const int* __restrict__ best, int a)
+{
+    const int b = best[a];
+    return b >= 0 && L[a].axis == 0 && best[b] == a;
+}
+
+#define PAIR_CHUNK 1024   // list entries whose matches are counted together
+
+__global__ void __launch_bounds__(256) k_pair_count(const ulm_loc2d* __restrict__ L, const int* __restrict__ n2d, int cap2d,
+                                                    const int* __restrict__ best, int* __restrict__ part)
+{
+    __shared__ int red[8];
+    const int n = min(*n2d, cap2d);
+    for (int c = blockIdx.x; c * PAIR_CHUNK < n; c += gridDim.x) {
+        int m = 0;
+#pragma unroll
+        for (int q = 0; q < PAIR_CHUNK; q += 256) {
+            const int a = c * PAIR_CHUNK + q + threadIdx.x;
+            if (a < n && pair_mutual(L, best, a)) ++m;
+        }
+        m = __reduce_add_sync(0xffffffffu, m);
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int t = 0;
+            for (int w = 0; w < 8; ++w) t += red[w];
+            part[c] = t;
         }
     }
-    match[a] = m;
 }
 
-__global__ void k_match_flags(const int* __restrict__ match, const int* __restrict__ n2d, int cap2d,
-                              int* __restrict__ flags)
+__global__ void __launch_bounds__(256) k_pair_write(const ulm_loc2d* __restrict__ L, const int* __restrict__ n2d, int cap2d,
+                                                    const int* __restrict__ best, const int* __restrict__ part,
+                                                    ulm_loc3d* __restrict__ out, int cap3d, int* __restrict__ n3d,
+                                                    unsigned* __restrict__ status)
 {
-    // every slot the scan reads, max(cap2d, 1) of them, is written (0 past the list)
-    const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= max(cap2d, 1)) return;
+    __shared__ int red[16];
+    constexpr int PER = PAIR_CHUNK / 256;
     const int n = min(*n2d, cap2d);
-    flags[a] = (a < n && match[a] >= 0) ? 1 : 0;
-}
-
-__global__ void k_pair_write(const ulm_loc2d* __restrict__ L, const int* __restrict__ n2d, int cap2d,
-                             const int* __restrict__ match, const int* __restrict__ off, ulm_loc3d* __restrict__ out,
-                             int cap3d, unsigned* __restrict__ status)
-{
-    const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    const int n = min(*n2d, cap2d);
-    if (a >= n || match[a] < 0) return;
-    const int dst = off[a];
-    if (dst >= cap3d) {
-        atomicOr(status, ST_CAPACITY);
+    if (n <= 0) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) *n3d = 0;
         return;
     }
-    const ulm_loc2d x = L[a], y = L[match[a]];
-    ulm_loc3d o;
-    o.frame = x.frame;
-    o.i_xz = a;
-    o.i_yz = match[a];
-    o.reserved = 0;
-    o.x = x.lat;
-    o.y = y.lat;
-    o.z = 0.5f * (x.z + y.z);
-    o.amp_xz = x.amp;
-    o.amp_yz = y.amp;
-    o.reserved2 = 0.f;
-    out[dst] = o;
+    for (int c = blockIdx.x; c * PAIR_CHUNK < n; c += gridDim.x) {
+        const int a0 = c * PAIR_CHUNK + PER * threadIdx.x;
+        unsigned m = 0u;
+#pragma unroll
+        for (int q = 0; q < PER; ++q)
+            if (a0 + q < n && pair_mutual(L, best, a0 + q)) m |= 1u << q;
+        int all;
+        int dst = block_offset(part, c, __popc(m), red, &all);
+        if (threadIdx.x == 0 && (c + 1) * PAIR_CHUNK >= n) *n3d = all;
+        while (m) {
+            const int a = a0 + __ffs(m) - 1, b = best[a];
+            m &= m - 1;
+            if (dst >= cap3d) {
+                atomicOr(status, ST_CAPACITY);
+                break;
+            }
+            const ulm_loc2d x = L[a], y = L[b];
+            ulm_loc3d o;
+            o.frame = x.frame;
+            o.i_xz = a;
+            o.i_yz = b;
+            o.reserved = 0;
+            o.x = x.lat;
+            o.y = y.lat;
+            o.z = 0.5f * (x.z + y.z);
+            o.amp_xz = x.amp;
+            o.amp_yz = y.amp;
+            o.reserved2 = 0.f;
+            out[dst++] = o;
+        }
+    }
 }
 
 }  // namespace
 
-// exclusive scan on the device; part: workspace of 2 * ceil(n_max / SCAN_CHUNK) long longs
-static rca_status device_scan(rca_handle* h, const int* cnt, int n_max, const int* n_dev, int cap_each, int* off,
-                              int* total_true, long long* part)
+// candidate slots of a detection, then their gather
+struct Slots {
+    ulm_loc2d* cand;
+    int *cnt, *part;
+    unsigned long long* total;
+};
+
+static rca_status slots_get(rca_handle* h, int nslots, Slots* o)
 {
-    const int nb = std::max(1, (n_max + SCAN_CHUNK - 1) / SCAN_CHUNK);
-    if (nb > 1024) return set_error(h, RCA_ERR_UNSUPPORTED, "scan over more than %d entries", 1024 * SCAN_CHUNK);
-    k_scan_part<<<nb, SCAN_THREADS, 0, h->stream>>>(cnt, n_max, n_dev, cap_each, part);
-    k_scan_top<<<1, 1024, 0, h->stream>>>(part, nb, n_max, n_dev, off, total_true);
-    k_scan_apply<<<nb, SCAN_THREADS, 0, h->stream>>>(cnt, n_max, n_dev, cap_each, part, off);
-    return cuda_check(h, cudaGetLastError(), "scan kernels");
+    rca_status st = RCA_OK;
+    o->cand = (ulm_loc2d*)ws_get(h, WS_CAND, (size_t)nslots * CAND_CAP * sizeof(ulm_loc2d), &st);
+    if (!o->cand) return st;
+    o->cnt = (int*)ws_get(h, WS_CANDCNT, (size_t)nslots * sizeof(int), &st);
+    if (!o->cnt) return st;
+    // the true total, then the chunks' kept totals
+    const size_t bytes = 16 + (size_t)((nslots + GATHER_SLOTS - 1) / GATHER_SLOTS) * sizeof(int);
+    char* p = (char*)ws_get(h, WS_SCAN, bytes, &st);
+    if (!p) return st;
+    o->total = reinterpret_cast<unsigned long long*>(p);
+    o->part = reinterpret_cast<int*>(p + 16);
+    return cuda_check(h, cudaMemsetAsync(p, 0, bytes, h->stream), "candidate totals");
+}
+
+static rca_status slots_gather(rca_handle* h, const Slots& o, int nslots, int nstrip, ulm_loc2d* out, int cap, int* n2d,
+                               int* poff, const float* A, const GeomDev& g)
+{
+    if (nslots > SCAN_MAX) return set_error(h, RCA_ERR_UNSUPPORTED, "scan over more than %d entries", SCAN_MAX);
+    k_gather<<<(nslots + GATHER_SLOTS - 1) / GATHER_SLOTS, 256, 0, h->stream>>>(
+        o.cand, o.cnt, o.part, o.total, nslots, nstrip, out, cap, n2d, poff, A, g.S, g.nz, g.N, h->d_status);
+    return cuda_check(h, cudaGetLastError(), "gather kernel");
+}
+
+// pairing on scratch: best [cap2d], part [chunks of PAIR_CHUNK]
+static rca_status pair_launch(rca_handle* h, const GeomDev& g, const ulm_loc2d* L, const int* n2d, int cap2d, int F,
+                              const int* poff, int* best, int* part, ulm_loc3d* out, int cap3d, int* n3d)
+{
+    const int nn = std::max(cap2d, 1);
+    if (nn > SCAN_MAX) return set_error(h, RCA_ERR_UNSUPPORTED, "scan over more than %d entries", SCAN_MAX);
+    // the list's length is known on the device only: grids of a few waves at most walk it
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int cap_blocks = 16 * sms;
+    const int nb = std::min(cap_blocks, (nn + 256 / PAIR_LANES - 1) / (256 / PAIR_LANES));
+    const int nc = std::min(cap_blocks, (nn + PAIR_CHUNK - 1) / PAIR_CHUNK);
+    k_pair_best<<<nb, 256, 0, h->stream>>>(L, n2d, cap2d, F, g.S, g.P, poff, best);
+    k_pair_count<<<nc, 256, 0, h->stream>>>(L, n2d, cap2d, best, part);
+    k_pair_write<<<nc, 256, 0, h->stream>>>(L, n2d, cap2d, best, part, out, cap3d, n3d, h->d_status);
+    return cuda_check(h, cudaGetLastError(), "pair kernels");
 }
 
 rca_status launch_enhance(rca_handle* h, const rca_tables* t, const void* planes, rca_dtype pt, int F, int enh,
@@ -899,13 +1022,9 @@ rca_status launch_detect2d(rca_handle* h, const rca_tables* t, const float* A, c
     const int nplanes = F * 2 * g.S;
     const int nslots = nplanes * nstrip;
     rca_status st = RCA_OK;
-    ulm_loc2d* cand = (ulm_loc2d*)ws_get(h, WS_CAND, (size_t)nslots * CAND_CAP * sizeof(ulm_loc2d), &st);
-    if (!cand) return st;
-    int* cnt = (int*)ws_get(h, WS_CANDCNT, (size_t)nslots * sizeof(int), &st);
-    if (!cnt) return st;
-    int* off = (int*)ws_get(h, WS_SCAN, (size_t)(nslots + 1) * sizeof(int), &st);
-    if (!off) return st;
     if (g.N % 2 != 0 || g.N > 256) return set_error(h, RCA_ERR_UNSUPPORTED, "NCC detection needs an even N <= 256");
+    Slots slots;
+    if ((st = slots_get(h, nslots, &slots)) != RCA_OK) return st;
     const int rin = NCC_RS + 2 + 2 * hh;
     // two buffers of amplitude rows (later the NCC rows, stride N + 1) + three
     // padded vertical-sum arrays of row pairs
@@ -920,21 +1039,23 @@ rca_status launch_detect2d(rca_handle* h, const rca_tables* t, const float* A, c
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaError_t e = cudaSuccess;
     switch (hh) {
-#define RCA_DETECT_LAUNCH(HV, NV)                                                                          \
+#define RCA_DETECT_LAUNCH(HV, NV, TV)                                                                      \
     do {                                                                                                   \
-        e = cudaFuncSetAttribute(k_detect<HV, NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+        auto kern = k_detect<HV, NV, TV>;                                                                  \
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);            \
         if (e != cudaSuccess) return cuda_check(h, e, "detect smem attribute");                          \
         int per_sm = 0;                                                                                    \
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_detect<HV, NV>, NCC_THREADS, smem);       \
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TV + 32, smem);                       \
         const dim3 grid((unsigned)std::max(1, std::min(nslots, std::max(1, per_sm) * sms)));               \
-        k_detect<HV, NV><<<grid, NCC_THREADS, smem, h->stream>>>(A, M, g.S, g.nz, g.N, nplanes, nc, cand, cnt, \
-                                                                 ncc_out, h->d_status);                   \
+        kern<<<grid, TV + 32, smem, h->stream>>>(A, M, g.S, g.nz, g.N, nplanes, nc, slots.cand, slots.cnt,      \
+                                            slots.part, slots.total, ncc_out, h->d_status);                \
     } while (0)
 #define RCA_DETECT_CASE(HV)                                                                                \
     case HV:                                                                                               \
-        if (g.N == 128) RCA_DETECT_LAUNCH(HV, 128);                                                        \
-        else if (g.N == 32) RCA_DETECT_LAUNCH(HV, 32);                                                     \
-        else RCA_DETECT_LAUNCH(HV, 0);                                                                     \
+        if (g.N == 128) RCA_DETECT_LAUNCH(HV, 128, NCC_THREADS);                                           \
+        else if (g.N == 32) RCA_DETECT_LAUNCH(HV, 32, NCC_THREADS / 2);                                    \
+        else if (g.N <= 64) RCA_DETECT_LAUNCH(HV, 0, NCC_THREADS / 2);                                     \
+        else RCA_DETECT_LAUNCH(HV, 0, NCC_THREADS);                                                        \
         break;
         RCA_DETECT_CASE(1)
         RCA_DETECT_CASE(2)
@@ -947,37 +1068,41 @@ rca_status launch_detect2d(rca_handle* h, const rca_tables* t, const float* A, c
 #undef RCA_DETECT_LAUNCH
     default: return set_error(h, RCA_ERR_INVALID_ARG, "NCC kernel length out of range");
     }
-    long long* part = (long long*)ws_get(h, WS_N2D, (size_t)2 * 1024 * sizeof(long long), &st);
-    if (!part) return st;
-    if ((st = device_scan(h, cnt, nslots, nullptr, CAND_CAP, off, n2d, part)) != RCA_OK) return st;
-    k_gather<<<(nslots + 7) / 8, 256, 0, h->stream>>>(cand, cnt, off, nslots, out, cap, A, g.S, g.nz, g.N,
-                                                      h->d_status);
-    if (plane_off) k_strip_to_plane<<<(nplanes + 1 + 255) / 256, 256, 0, h->stream>>>(off, nstrip, nplanes, plane_off);
-    return cuda_check(h, cudaGetLastError(), "detect kernels");
+    if ((st = cuda_check(h, cudaGetLastError(), "detect kernel")) != RCA_OK) return st;
+    return slots_gather(h, slots, nslots, nstrip, out, cap, n2d, plane_off, A, g);
 }
 
 rca_status launch_pair3d(rca_handle* h, const rca_tables* t, const ulm_loc2d* L, const int* n2d, int cap2d, int F,
-                         ulm_loc3d* out, int cap3d, int* n3d)
+                         ulm_loc3d* out, int cap3d, int* n3d, const int* plane_off)
 {
     const GeomDev& g = t->gd;
     const int nplanes = F * 2 * g.S;
     rca_status st = RCA_OK;
-    int* poff = (int*)ws_get(h, WS_PLANEOFF, (size_t)(nplanes + 1) * sizeof(int), &st);
-    if (!poff) return st;
     const int nn = std::max(cap2d, 1);
-    int* match = (int*)ws_get(h, WS_FLAGS, (size_t)nn * 2 * sizeof(int), &st);
-    if (!match) return st;
-    int* flags = match + nn;
-    int* off = (int*)ws_get(h, WS_MISC, (size_t)(nn + 1) * sizeof(int), &st);
-    if (!off) return st;
-    k_list_plane_offsets<<<(nplanes + 1 + 255) / 256, 256, 0, h->stream>>>(L, n2d, cap2d, g.S, nplanes, poff);
-    k_pair_match<<<(nn + 255) / 256, 256, 0, h->stream>>>(L, n2d, cap2d, g.S, g.P, poff, match);
-    k_match_flags<<<(nn + 255) / 256, 256, 0, h->stream>>>(match, n2d, cap2d, flags);
-    long long* part = (long long*)ws_get(h, WS_N2D, (size_t)2 * 1024 * sizeof(long long), &st);
+    int* best = (int*)ws_get(h, WS_FLAGS, (size_t)nn * sizeof(int), &st);
+    if (!best) return st;
+    int* part = (int*)ws_get(h, WS_MISC, (size_t)((nn + PAIR_CHUNK - 1) / PAIR_CHUNK) * sizeof(int), &st);
     if (!part) return st;
-    if ((st = device_scan(h, flags, nn, n2d, 0, off, n3d, part)) != RCA_OK) return st;
-    k_pair_write<<<(nn + 255) / 256, 256, 0, h->stream>>>(L, n2d, cap2d, match, off, out, cap3d, h->d_status);
-    return cuda_check(h, cudaGetLastError(), "pair kernels");
+    if (!plane_off) {
+        int* poff = (int*)ws_get(h, WS_PLANEOFF, (size_t)(nplanes + 1) * sizeof(int), &st);
+        if (!poff) return st;
+        k_list_plane_offsets<<<(nplanes + 1 + 255) / 256, 256, 0, h->stream>>>(L, n2d, cap2d, g.S, nplanes, poff);
+        plane_off = poff;
+    }
+    return pair_launch(h, g, L, n2d, cap2d, F, plane_off, best, part, out, cap3d, n3d);
+}
+
+// detection and pairing of one ensemble: the detection's gather writes the plane
+// offsets that the pairing needs
+rca_status launch_detect_pair(rca_handle* h, const rca_tables* t, const float* A, const float* M, int F,
+                              const ulm_params* prm, ulm_loc2d* out2d, int cap2d, int* n2d, ulm_loc3d* out3d, int cap3d,
+                              int* n3d)
+{
+    rca_status st = RCA_OK;
+    int* poff = (int*)ws_get(h, WS_PLANEOFF, ((size_t)F * 2 * t->gd.S + 1) * sizeof(int), &st);
+    if (!poff) return st;
+    if ((st = launch_detect2d(h, t, A, M, F, prm, out2d, cap2d, n2d, nullptr, poff)) != RCA_OK) return st;
+    return launch_pair3d(h, t, out2d, n2d, cap2d, F, out3d, cap3d, n3d, poff);
 }
 
 // ---------------------------------------------------------------------------
@@ -997,22 +1122,18 @@ rca_status launch_pair3d(rca_handle* h, const rca_tables* t, const ulm_loc2d* L,
 // process (a device reset makes the kept address stale; rca.h says so).
 //
 // Nothing in it needs clearing between calls: each call writes every entry
-// it reads (plane offsets for all planes, flags for all list slots, match
-// indices and scan offsets for all live entries, one partial per scan
-// chunk), so the previous call's contents are never seen.
+// it reads (plane offsets for all planes, partners for all live entries, one
+// count per live chunk), so the previous call's contents are never seen.
 // ---------------------------------------------------------------------------
 namespace {
 
 constexpr size_t na_round(size_t b) { return (b + 255) & ~(size_t)255; }
-constexpr int NA_CHUNKS = (ULM_PAIR3D_NOALLOC_MAX_2D + SCAN_CHUNK - 1) / SCAN_CHUNK;
+constexpr int NA_CHUNKS = (ULM_PAIR3D_NOALLOC_MAX_2D + PAIR_CHUNK - 1) / PAIR_CHUNK;
 constexpr size_t NA_POFF = 0;
-constexpr size_t NA_MATCH = NA_POFF + na_round((size_t)(ULM_PAIR3D_NOALLOC_MAX_PLANES + 1) * sizeof(int));
-constexpr size_t NA_FLAGS = NA_MATCH + na_round((size_t)ULM_PAIR3D_NOALLOC_MAX_2D * sizeof(int));
-constexpr size_t NA_OFF = NA_FLAGS + na_round((size_t)ULM_PAIR3D_NOALLOC_MAX_2D * sizeof(int));
-constexpr size_t NA_PART = NA_OFF + na_round((size_t)(ULM_PAIR3D_NOALLOC_MAX_2D + 1) * sizeof(int));
-constexpr size_t NA_BYTES = NA_PART + na_round((size_t)2 * NA_CHUNKS * sizeof(long long));
-static_assert(NA_BYTES == ULM_PAIR3D_NOALLOC_SCRATCH_BYTES, "scratch size stated in rca.h is stale");
-static_assert(NA_CHUNKS <= 1024, "device_scan handles at most 1024 chunks");
+constexpr size_t NA_BEST = NA_POFF + na_round((size_t)(ULM_PAIR3D_NOALLOC_MAX_PLANES + 1) * sizeof(int));
+constexpr size_t NA_PART = NA_BEST + na_round((size_t)ULM_PAIR3D_NOALLOC_MAX_2D * sizeof(int));
+constexpr size_t NA_BYTES = ULM_PAIR3D_NOALLOC_SCRATCH_BYTES;   // the size that rca.h states
+static_assert(NA_PART + na_round((size_t)NA_CHUNKS * sizeof(int)) <= NA_BYTES, "scratch size stated in rca.h is too small");
 
 constexpr int NA_MAX_DEVICES = 64;
 
@@ -1055,18 +1176,11 @@ rca_status launch_pair3d_noalloc(rca_handle* h, const rca_tables* t, const ulm_l
     rca_status st = pair_scratch(h, &base);
     if (st != RCA_OK) return st;
     int* poff = reinterpret_cast<int*>(base + NA_POFF);
-    int* match = reinterpret_cast<int*>(base + NA_MATCH);
-    int* flags = reinterpret_cast<int*>(base + NA_FLAGS);
-    int* off = reinterpret_cast<int*>(base + NA_OFF);
-    long long* part = reinterpret_cast<long long*>(base + NA_PART);
-    const int nn = std::max(cap2d, 1);
+    int* best = reinterpret_cast<int*>(base + NA_BEST);
+    int* part = reinterpret_cast<int*>(base + NA_PART);
     const int np = (int)nplanes;
     k_list_plane_offsets<<<(np + 1 + 255) / 256, 256, 0, h->stream>>>(L, n2d, cap2d, g.S, np, poff);
-    k_pair_match<<<(nn + 255) / 256, 256, 0, h->stream>>>(L, n2d, cap2d, g.S, g.P, poff, match);
-    k_match_flags<<<(nn + 255) / 256, 256, 0, h->stream>>>(match, n2d, cap2d, flags);
-    if ((st = device_scan(h, flags, nn, n2d, 0, off, n3d, part)) != RCA_OK) return st;
-    k_pair_write<<<(nn + 255) / 256, 256, 0, h->stream>>>(L, n2d, cap2d, match, off, out, cap3d, h->d_status);
-    return cuda_check(h, cudaGetLastError(), "pair kernels (no-alloc)");
+    return pair_launch(h, g, L, n2d, cap2d, F, poff, best, part, out, cap3d, n3d);
 }
 
 rca_status launch_detect_map(rca_handle* h, const rca_tables* t, const float* map, int up, const float* A, const float* M,
@@ -1078,23 +1192,16 @@ rca_status launch_detect_map(rca_handle* h, const rca_tables* t, const float* ma
     const int nplanes = F * 2 * g.S;
     const int nslots = nplanes * nstrip;
     rca_status st = RCA_OK;
-    ulm_loc2d* cand = (ulm_loc2d*)ws_get(h, WS_CAND, (size_t)nslots * CAND_CAP * sizeof(ulm_loc2d), &st);
-    if (!cand) return st;
-    int* cnt = (int*)ws_get(h, WS_CANDCNT, (size_t)nslots * sizeof(int), &st);
-    if (!cnt) return st;
-    int* off = (int*)ws_get(h, WS_SCAN, (size_t)(nslots + 1) * sizeof(int), &st);
-    if (!off) return st;
-    long long* part = (long long*)ws_get(h, WS_N2D, (size_t)2 * 1024 * sizeof(long long), &st);
-    if (!part) return st;
+    Slots slots;
+    if ((st = slots_get(h, nslots, &slots)) != RCA_OK) return st;
     // the strip's rows plus the candidate bitmap of its pixels
     const size_t smem = (size_t)(DET_RS + 2) * W4 * sizeof(float) + (size_t)((DET_RS * W4 + 31) / 32) * sizeof(unsigned);
     if (smem > 200 * 1024) return set_error(h, RCA_ERR_UNSUPPORTED, "map rows of %d fine pixels exceed shared memory", W4);
     cudaError_t e = cudaFuncSetAttribute(k_detect_map, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_check(h, e, "detect_map smem attribute");
     dim3 grid(nstrip, nplanes);
-    k_detect_map<<<grid, 256, smem, h->stream>>>(map, up, A, M, g.S, g.nz, g.N, score_min, alpha, cand, cnt, h->d_status);
-    if ((st = device_scan(h, cnt, nslots, nullptr, CAND_CAP, off, n2d, part)) != RCA_OK) return st;
-    k_gather<<<(nslots + 7) / 8, 256, 0, h->stream>>>(cand, cnt, off, nslots, out, cap, nullptr, 0, 0, 0,
-                                                      h->d_status);
-    return cuda_check(h, cudaGetLastError(), "detect_map kernels");
+    k_detect_map<<<grid, 256, smem, h->stream>>>(map, up, A, M, g.S, g.nz, g.N, score_min, alpha, slots.cand, slots.cnt,
+                                                 slots.part, slots.total, h->d_status);
+    if ((st = cuda_check(h, cudaGetLastError(), "detect_map kernel")) != RCA_OK) return st;
+    return slots_gather(h, slots, nslots, nstrip, out, cap, n2d, nullptr, nullptr, g);
 }

@@ -45,9 +45,8 @@ enum WsSlot {
     WS_CAND,       // ulm_loc2d [strips][CAND_CAP]
     WS_CANDCNT,    // int [strips]
     WS_PLANEOFF,   // int [planes + 1]
-    WS_FLAGS,      // int [n]
-    WS_SCAN,       // int [n + 1]
-    WS_N2D,        // int [1]
+    WS_FLAGS,      // pairing partner of every list entry
+    WS_SCAN,       // totals of the candidate slots
     WS_MISC,       // small scratch
     WS_TRACK,      // tracking: frame offsets, links, flags, positions, per-localisation tracks
     WS_MOTION,     // motion estimation: twiddles, row spectra, reference spectrum, correlations
@@ -266,7 +265,10 @@ rca_status launch_detect2d(rca_handle* h, const rca_tables* t, const float* A, c
 rca_status launch_detect_map(rca_handle* h, const rca_tables* t, const float* map, int up, const float* A, const float* M,
                              int F, float score_min, float alpha, ulm_loc2d* out, int cap, int* n2d);
 rca_status launch_pair3d(rca_handle* h, const rca_tables* t, const ulm_loc2d* L, const int* n2d, int cap2d,
-                         int F, ulm_loc3d* out, int cap3d, int* n3d);
+                         int F, ulm_loc3d* out, int cap3d, int* n3d, const int* plane_off);
+rca_status launch_detect_pair(rca_handle* h, const rca_tables* t, const float* A, const float* M, int F,
+                              const ulm_params* prm, ulm_loc2d* out2d, int cap2d, int* n2d, ulm_loc3d* out3d, int cap3d,
+                              int* n3d);
 rca_status launch_fp32_probe(rca_handle* h, int packed, int iters, float* sink, double* flops);
 rca_status launch_pair3d_noalloc(rca_handle* h, const rca_tables* t, const ulm_loc2d* L, const int* n2d,
                                  int cap2d, int F, ulm_loc3d* out, int cap3d, int* n3d);
