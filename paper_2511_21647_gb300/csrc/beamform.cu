@@ -10,6 +10,7 @@ namespace {
 __global__ void __launch_bounds__(256) k_mean(const void* __restrict__ rf, int rf_t, const float* __restrict__ scale,
                                               int F, int ns, int ncol, float* __restrict__ mean)
 {
+    grid_wait();
     mean_body(blockIdx.x, rf, rf_t, scale, F, ns, ncol, mean);
 }
 
@@ -18,6 +19,7 @@ __global__ void __launch_bounds__(256, 4) k_demod(const void* __restrict__ rf, c
                                                   const float* __restrict__ mean, const float2* __restrict__ mix,
                                                   Fir fir, int nt, int E, int ns, void* __restrict__ iq, int iq_t)
 {
+    grid_wait();
     __shared__ float2 xs[DM_NE * DM_PITCH];
     demod_body<RT>(blockIdx.x, blockIdx.y, blockIdx.z, xs, rf, scale, mean, mix, fir, nt, E, ns, iq, iq_t);
 }
@@ -29,6 +31,7 @@ __global__ void __launch_bounds__(256, 2) k_stage1(GeomDev g, const void* __rest
                                                 int dc, int n_tiles, int nch, int ring, float2* __restrict__ slices,
                                                 unsigned* __restrict__ status)
 {
+    grid_wait();
     extern __shared__ __align__(128) unsigned char smraw[];
     __shared__ uint64_t bars[2];
     stage1_body<TS, MAXR, true, PAIR>(blockIdx.x, blockIdx.y, blockIdx.z, smraw, bars, g, iq, rtab, rblk, dmax, chunks, zt,
@@ -44,6 +47,7 @@ __global__ void __launch_bounds__(S2_THREADS, 3) k_stage2(GeomDev g, const float
                                                        int rows, int smin0, int smin1, void* __restrict__ planes,
                                                        int pt, unsigned* __restrict__ status)
 {
+    grid_wait();
     extern __shared__ __align__(128) unsigned char smraw[];
     __shared__ uint64_t bar;
     stage2_body<TM, US>(blockIdx.x, blockIdx.y, blockIdx.z & 1, blockIdx.z >> 1, smraw, &bar, g, slices, sfl, sfr, lw, rot,
@@ -177,17 +181,17 @@ rca_status launch_ingest(rca_handle* h, const rca_tables* t, const void* rf, rca
         const int ncol = nt * g.N * g.ns;
         mean = (float*)ws_get(h, WS_MEAN, (size_t)ncol * sizeof(float), &st);
         if (!mean) return st;
-        k_mean<<<(ncol / 4 + 255) / 256, 256, 0, h->stream>>>(rf, rf_t, scale, F, g.ns, ncol, mean);
+        launch_chain(k_mean, dim3((ncol / 4 + 255) / 256), dim3(256), 0, h->stream, rf, rf_t, scale, F, g.ns, ncol, mean);
     }
     Fir fir;
     for (int q = 0; q < 31; ++q) fir.h[q] = t->fir[q];
     dim3 grid((g.ns + DM_NT - 1) / DM_NT, (g.N + DM_NE - 1) / DM_NE, F * nt);
     if (rf_t == RCA_F32)
-        k_demod<RCA_F32><<<grid, 256, 0, h->stream>>>(rf, scale, mean, t->mix, fir, nt, g.N, g.ns, iq, iq_t);
+        launch_chain(k_demod<RCA_F32>, grid, dim3(256), 0, h->stream, rf, scale, mean, t->mix, fir, nt, g.N, g.ns, iq, iq_t);
     else if (rf_t == RCA_F16)
-        k_demod<RCA_F16><<<grid, 256, 0, h->stream>>>(rf, scale, mean, t->mix, fir, nt, g.N, g.ns, iq, iq_t);
+        launch_chain(k_demod<RCA_F16>, grid, dim3(256), 0, h->stream, rf, scale, mean, t->mix, fir, nt, g.N, g.ns, iq, iq_t);
     else
-        k_demod<RCA_I16><<<grid, 256, 0, h->stream>>>(rf, scale, mean, t->mix, fir, nt, g.N, g.ns, iq, iq_t);
+        launch_chain(k_demod<RCA_I16>, grid, dim3(256), 0, h->stream, rf, scale, mean, t->mix, fir, nt, g.N, g.ns, iq, iq_t);
     return cuda_check(h, cudaGetLastError(), "ingest kernels");
 }
 
@@ -203,7 +207,7 @@ static rca_status stage1_launch(rca_handle* h, const rca_tables* t, const void* 
     if (e != cudaSuccess) return cuda_check(h, e, "stage1 smem attribute");
     dim3 grid(p.n_tiles, 2 * g.K, F);
     const unsigned char* rtab = std::is_same<TS, __half2>::value ? p.d_rec16 : p.d_rec32;
-    kern<<<grid, threads, smem, h->stream>>>(g, iq, rtab, p.rblk, t->dmax, p.d_chunks, p.zt, p.dc, p.n_tiles, p.nch,
+    launch_chain(kern, grid, dim3(threads), smem, h->stream, g, iq, rtab, p.rblk, t->dmax, p.d_chunks, p.zt, p.dc, p.n_tiles, p.nch,
                                              p.ring, slices, h->d_status);
     return cuda_check(h, cudaGetLastError(), "stage1 kernel");
 }
@@ -256,7 +260,7 @@ static rca_status stage2_launch(rca_handle* h, const rca_tables* t, const float2
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_check(h, e, "stage2 smem attribute");
     dim3 grid(t->s2.n_tiles, (g.N + GW - 1) / GW, 2 * F);
-    kern<<<grid, S2_THREADS, smem, h->stream>>>(g, slices, t->s2_sfl, t->s2_sfr, t->s2_lw, t->s2_rot, t->s2_coefr,
+    launch_chain(kern, grid, dim3(S2_THREADS), smem, h->stream, g, slices, t->s2_sfl, t->s2_sfr, t->s2_lw, t->s2_rot, t->s2_coefr,
                                                 t->s2_c2r, t->s2_tmin, t->T, t->s2_iA, t->s2_iB, t->s2.zp, t->s2.rows,
                                                 t->s2.smin[0], t->s2.smin[1], planes, (int)pt, h->d_status);
     return cuda_check(h, cudaGetLastError(), "stage2 kernel");

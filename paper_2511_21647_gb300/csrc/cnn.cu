@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(128) k_conv_tc(const __nv_bfloat16* __restrict
                                                  const __nv_bfloat16* __restrict__ mask, int B, int H, int W,
                                                  __nv_bfloat16* __restrict__ out, unsigned* __restrict__ status)
 {
+    grid_wait();
     static_assert(CIN % 16 == 0 && COUT % 16 == 0 && COUT <= 32, "shapes of the 3x3 layers");
     constexpr int KC = CIN / 8, NG = COUT / 8;
     constexpr int TAPB = KC * NG * 128;                 // bytes of one tap's weights
@@ -361,6 +362,7 @@ template <int COUT>
 __global__ void __launch_bounds__(288, 3) k_wgrad_mma(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ dy,
                                                       int B, int H, int W, float* __restrict__ part)
 {
+    grid_wait();
     constexpr int MT = COUT / 16, DC = COUT / 8, DS = WG_DS(COUT), XOFF = CONV_TH * CONV_TW * DS, HW2 = CONV_TW + 2;
     constexpr int N = 9 * CNN_C;
     extern __shared__ __align__(16) unsigned char smraw[];   // [2][dY tile, X tile with halo]
@@ -455,6 +457,7 @@ __global__ void __launch_bounds__(288, 3) k_wgrad_mma(const __nv_bfloat16* __res
 __global__ void __launch_bounds__(256) k_wgrad1(const float* __restrict__ x, const __nv_bfloat16* __restrict__ dy, int rows,
                                                 int H, int W, float* __restrict__ part)
 {
+    grid_wait();
     __shared__ float red[8][CNN_C * 10];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float s[10];
@@ -507,6 +510,7 @@ struct GradSums {
 
 __global__ void __launch_bounds__(256) k_reduce_grads(const GradSums g)
 {
+    grid_wait();
     __shared__ float red[8][32];
     int seg = 0;
     while (seg < 4 && (int)blockIdx.x >= g.block0[seg + 1]) ++seg;
@@ -539,6 +543,7 @@ template <bool ALIGNED>
 __global__ void __launch_bounds__(256) k_loss(const float* __restrict__ heat, const float* __restrict__ target, int rows,
                                               int W, float scale, __nv_bfloat16* __restrict__ dz, float* __restrict__ part)
 {
+    grid_wait();
     __shared__ float red[8];
     const unsigned np = (unsigned)rows * W;                    // within the network's capacity, an int
     float s = 0.f;
@@ -585,6 +590,7 @@ struct PackedWeights {
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ gr, float* __restrict__ m, float* __restrict__ v,
                        const PackedWeights w, float lr_t, float b1, float b2, float eps_t)
 {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= w.lay.total) return;
     const float g = gr[i];
@@ -712,7 +718,7 @@ static rca_status conv_launch(ulm_cnn* c, const __nv_bfloat16* x, const __nv_bfl
     if (e != cudaSuccess) return cuda_check(c->h, e, "conv smem attribute");
     const int ntiles = B * ((H + CONV_TH - 1) / CONV_TH) * ((W + CONV_TW - 1) / CONV_TW);
     const int grid = std::min(ntiles, c->grid_conv_tc);
-    kern<<<grid, 128, smem, c->h->stream>>>(x, w, mask, B, H, W, out, c->h->d_status);
+    launch_chain(kern, dim3(grid), dim3(128), smem, c->h->stream, x, w, mask, B, H, W, out, c->h->d_status);
     return cuda_check(c->h, cudaGetLastError(), "conv kernel");
 }
 
@@ -727,7 +733,7 @@ static rca_status wgrad_launch(ulm_cnn* c, const __nv_bfloat16* x, const __nv_bf
     if (e != cudaSuccess) return cuda_check(c->h, e, "wgrad smem attribute");
     const int ntiles = B * ((H + CONV_TH - 1) / CONV_TH) * ((W + CONV_TW - 1) / CONV_TW);
     sums.part[l] = c->part + at, sums.nparts[l] = std::min(ntiles, c->grid_wgrad), sums.len[l] = COUT * 9 * CNN_C + COUT;
-    kern<<<sums.nparts[l], 288, smem, c->h->stream>>>(x, dy, B, H, W, c->part + at);
+    launch_chain(kern, dim3(sums.nparts[l]), dim3(288), smem, c->h->stream, x, dy, B, H, W, c->part + at);
     at += (size_t)c->grid_wgrad * sums.len[l];
     return cuda_check(c->h, cudaGetLastError(), "wgrad kernel");
 }
@@ -747,7 +753,7 @@ static rca_status cnn_forward(ulm_cnn* c, const float* A, const float* M, int pp
     auto kern = k_cnn_stream<KEEP>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, StreamSmem::bytes);
     if (e != cudaSuccess) return cuda_check(c->h, e, "cnn smem attribute");
-    kern<<<std::min(g.plan.nruns, sms), ST_THREADS, StreamSmem::bytes, c->h->stream>>>(g);
+    launch_chain(kern, dim3(std::min(g.plan.nruns, sms)), dim3(ST_THREADS), StreamSmem::bytes, c->h->stream, g);
     return cuda_check(c->h, cudaGetLastError(), "cnn forward");
 }
 
@@ -896,9 +902,9 @@ extern "C" rca_status ulm_cnn_train_step(ulm_cnn* c, const float* A, const float
     const int lgrid = (int)std::min<size_t>((px + 255) / 256, CNN_LOSS_BLOCKS);
     float* lpart = c->part + (c->part_len - CNN_LOSS_BLOCKS);
     if ((reinterpret_cast<uintptr_t>(target) & 15) == 0)
-        k_loss<true><<<lgrid, 256, 0, s>>>(c->heat, target, B * H, W, 2.0f / n, c->gz, lpart);
+        launch_chain(k_loss<true>, dim3(lgrid), dim3(256), 0, s, c->heat, target, B * H, W, 2.0f / n, c->gz, lpart);
     else
-        k_loss<false><<<lgrid, 256, 0, s>>>(c->heat, target, B * H, W, 2.0f / n, c->gz, lpart);
+        launch_chain(k_loss<false>, dim3(lgrid), dim3(256), 0, s, c->heat, target, B * H, W, 2.0f / n, c->gz, lpart);
     // layer 4: dW4 from (a3, dz); dgrad -> g3 masked by a3 > 0
     if ((st = wgrad_launch<CNN_UP * CNN_UP>(c, c->a3, c->gz, B, H, W, 3, sums, at)) != RCA_OK) return st;
     if ((st = conv_launch<CNN_UP * CNN_UP, CNN_C>(c, c->gz, c->wfl[3], c->a3, B, H, W, c->g3)) != RCA_OK) return st;
@@ -910,12 +916,12 @@ extern "C" rca_status ulm_cnn_train_step(ulm_cnn* c, const float* A, const float
     if ((st = conv_launch<CNN_C, CNN_C>(c, c->g2, c->wfl[1], c->a1, B, H, W, c->g1)) != RCA_OK) return st;
     // layer 1 (FP32)
     sums.part[0] = c->part + at, sums.nparts[0] = std::min(c->grid_wgrad, (B * H + 7) / 8), sums.len[0] = CNN_C * 10;
-    k_wgrad1<<<sums.nparts[0], 256, 0, s>>>(c->x0, c->g1, B * H, H, W, c->part + at);
+    launch_chain(k_wgrad1, dim3(sums.nparts[0]), dim3(256), 0, s, c->x0, c->g1, B * H, H, W, c->part + at);
     // every layer's sums and the loss
     sums.part[4] = lpart, sums.nparts[4] = lgrid, sums.len[4] = 1, sums.out[4] = loss_dev, sums.scale[4] = 1.0f / n;
     for (int l = 0; l < 4; ++l) sums.out[l] = c->grads + L.w[l], sums.scale[l] = 1.f;
     for (int l = 0; l < 5; ++l) sums.block0[l + 1] = sums.block0[l] + (sums.len[l] + 31) / 32;
-    k_reduce_grads<<<sums.block0[5], 256, 0, s>>>(sums);
+    launch_chain(k_reduce_grads, dim3(sums.block0[5]), dim3(256), 0, s, sums);
     if ((st = cuda_check(c->h, cudaGetLastError(), "backward kernels")) != RCA_OK) return st;
     if (!apply_update) return RCA_OK;
     c->step += 1;
@@ -927,7 +933,7 @@ extern "C" rca_status ulm_cnn_train_step(ulm_cnn* c, const float* A, const float
     PackedWeights w{};
     w.lay = L;
     for (int l = 1; l < 4; ++l) w.fwd[l] = c->wbf[l], w.flip[l] = c->wfl[l];
-    k_adam<<<(L.total + 255) / 256, 256, 0, s>>>(c->params, c->grads, c->m, c->v, w, lr_t, (float)b1, (float)b2, eps_t);
+    launch_chain(k_adam, dim3((L.total + 255) / 256), dim3(256), 0, s, c->params, c->grads, c->m, c->v, w, lr_t, (float)b1, (float)b2, eps_t);
     return cuda_check(c->h, cudaGetLastError(), "adam");
 }
 

@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_cnn_stream(const StreamArgs g
     const int strip = issuer ? wid - 8 * ST_STRIPS : wid / 4 % ST_STRIPS, warp = wid & 3;
     const int lane = threadIdx.x & 31, tid = 32 * warp + lane;
     const int H = g.H, W = g.W;
+    grid_wait();
     st_stage_weights<32>(sms + StreamSmem::w2, g.w2);
     st_stage_weights<32>(sms + StreamSmem::w3, g.w3);
     st_stage_weights<16>(sms + StreamSmem::w4, g.w4);

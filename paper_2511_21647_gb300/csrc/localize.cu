@@ -35,6 +35,7 @@ template <int PT>
 __global__ void __launch_bounds__(256) k_enhance(const void* __restrict__ planes, int F, int S, size_t plane_sz,
                                                  int enh, int tf, float* __restrict__ A, unsigned* __restrict__ M)
 {
+    grid_wait();
     extern __shared__ unsigned mx[];  // [tf] maxima of this chunk's frames
     const int t0 = blockIdx.y * tf, t1 = min(F, t0 + tf);
     for (int t = threadIdx.x; t < t1 - t0; t += blockDim.x) mx[t] = 0u;
@@ -241,6 +242,7 @@ __global__ void __launch_bounds__(NT + 32, 512 / NT) k_detect(const float* __res
         }
     }
     __syncthreads();
+    grid_wait();
     if (threadIdx.x >= NT) {
         // ---- serving warp
         const int lane = threadIdx.x - NT;
@@ -533,6 +535,7 @@ __global__ void __launch_bounds__(256) k_detect_map(const float* __restrict__ ma
                                                     int* __restrict__ part, unsigned long long* __restrict__ total,
                                                     unsigned* __restrict__ status)
 {
+    grid_wait();
     extern __shared__ __align__(128) float smf[];
     __shared__ int wsum[32];
     __shared__ uint64_t bar;
@@ -688,6 +691,7 @@ __global__ void __launch_bounds__(256) k_gather(const ulm_loc2d* __restrict__ ca
                                                 int* __restrict__ n_out, int* __restrict__ poff, const float* __restrict__ A,
                                                 int S, int nz, int N, unsigned* __restrict__ status)
 {
+    grid_wait();
     static_assert(GATHER_SLOTS == 256, "a thread per slot");
     __shared__ int red[16], off[GATHER_SLOTS + 1];
     const int s0 = blockIdx.x * GATHER_SLOTS, s = s0 + threadIdx.x;
@@ -728,6 +732,7 @@ __device__ __forceinline__ int plane_key(const ulm_loc2d& e, int S) { return (e.
 __global__ void k_list_plane_offsets(const ulm_loc2d* __restrict__ L, const int* __restrict__ n2d, int cap2d, int S,
                                      int nplanes, int* __restrict__ poff)
 {
+    grid_wait();
     int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p > nplanes) return;
     int n = min(*n2d, cap2d);
@@ -792,6 +797,7 @@ __device__ __forceinline__ bool pair_better(float a, int p, float pa, int q, flo
 __global__ void __launch_bounds__(256) k_pair_best(const ulm_loc2d* __restrict__ L, const int* __restrict__ n2d, int cap2d,
                                                    int F, int S, int P, const int* __restrict__ poff, int* __restrict__ best)
 {
+    grid_wait();
     const int n = min(*n2d, cap2d), sub = threadIdx.x % PAIR_LANES;
     constexpr int PER = 256 / PAIR_LANES;
     for (int a0 = blockIdx.x * PER; a0 < n; a0 += gridDim.x * PER) {
@@ -840,6 +846,7 @@ __device__ __forceinline__ bool pair_mutual(const ulm_loc2d* __restrict__ L, con
 __global__ void __launch_bounds__(256) k_pair_count(const ulm_loc2d* __restrict__ L, const int* __restrict__ n2d, int cap2d,
                                                     const int* __restrict__ best, int* __restrict__ part)
 {
+    grid_wait();
     __shared__ int red[8];
     const int n = min(*n2d, cap2d);
     for (int c = blockIdx.x; c * PAIR_CHUNK < n; c += gridDim.x) {
@@ -866,6 +873,7 @@ __global__ void __launch_bounds__(256) k_pair_write(const ulm_loc2d* __restrict_
                                                     ulm_loc3d* __restrict__ out, int cap3d, int* __restrict__ n3d,
                                                     unsigned* __restrict__ status)
 {
+    grid_wait();
     __shared__ int red[16];
     constexpr int PER = PAIR_CHUNK / 256;
     const int n = min(*n2d, cap2d);
@@ -935,7 +943,7 @@ static rca_status slots_gather(rca_handle* h, const Slots& o, int nslots, int ns
                                int* poff, const float* A, const GeomDev& g)
 {
     if (nslots > SCAN_MAX) return set_error(h, RCA_ERR_UNSUPPORTED, "scan over more than %d entries", SCAN_MAX);
-    k_gather<<<(nslots + GATHER_SLOTS - 1) / GATHER_SLOTS, 256, 0, h->stream>>>(
+    launch_chain(k_gather, dim3((nslots + GATHER_SLOTS - 1) / GATHER_SLOTS), dim3(256), 0, h->stream, 
         o.cand, o.cnt, o.part, o.total, nslots, nstrip, out, cap, n2d, poff, A, g.S, g.nz, g.N, h->d_status);
     return cuda_check(h, cudaGetLastError(), "gather kernel");
 }
@@ -953,9 +961,9 @@ static rca_status pair_launch(rca_handle* h, const GeomDev& g, const ulm_loc2d* 
     const int cap_blocks = 16 * sms;
     const int nb = std::min(cap_blocks, (nn + 256 / PAIR_LANES - 1) / (256 / PAIR_LANES));
     const int nc = std::min(cap_blocks, (nn + PAIR_CHUNK - 1) / PAIR_CHUNK);
-    k_pair_best<<<nb, 256, 0, h->stream>>>(L, n2d, cap2d, F, g.S, g.P, poff, best);
-    k_pair_count<<<nc, 256, 0, h->stream>>>(L, n2d, cap2d, best, part);
-    k_pair_write<<<nc, 256, 0, h->stream>>>(L, n2d, cap2d, best, part, out, cap3d, n3d, h->d_status);
+    launch_chain(k_pair_best, dim3(nb), dim3(256), 0, h->stream, L, n2d, cap2d, F, g.S, g.P, poff, best);
+    launch_chain(k_pair_count, dim3(nc), dim3(256), 0, h->stream, L, n2d, cap2d, best, part);
+    launch_chain(k_pair_write, dim3(nc), dim3(256), 0, h->stream, L, n2d, cap2d, best, part, out, cap3d, n3d, h->d_status);
     return cuda_check(h, cudaGetLastError(), "pair kernels");
 }
 
@@ -986,7 +994,7 @@ rca_status launch_enhance(rca_handle* h, const rca_tables* t, const void* planes
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_check(h, e, "enhance smem attribute");
     dim3 grid(pblocks, (unsigned)((F + tf - 1) / tf));
-    kern<<<grid, 256, smem, h->stream>>>(planes, F, g.S, plane_sz, enh, tf, A, reinterpret_cast<unsigned*>(M));
+    launch_chain(kern, grid, dim3(256), smem, h->stream, planes, F, g.S, plane_sz, enh, tf, A, reinterpret_cast<unsigned*>(M));
     return cuda_check(h, cudaGetLastError(), "enhance kernel");
 }
 
@@ -1047,7 +1055,7 @@ rca_status launch_detect2d(rca_handle* h, const rca_tables* t, const float* A, c
         int per_sm = 0;                                                                                    \
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TV + 32, smem);                       \
         const dim3 grid((unsigned)std::max(1, std::min(nslots, std::max(1, per_sm) * sms)));               \
-        kern<<<grid, TV + 32, smem, h->stream>>>(A, M, g.S, g.nz, g.N, nplanes, nc, slots.cand, slots.cnt,      \
+        launch_chain(kern, grid, dim3(TV + 32), smem, h->stream, A, M, g.S, g.nz, g.N, nplanes, nc, slots.cand, slots.cnt,      \
                                             slots.part, slots.total, ncc_out, h->d_status);                \
     } while (0)
 #define RCA_DETECT_CASE(HV)                                                                                \
@@ -1086,7 +1094,7 @@ rca_status launch_pair3d(rca_handle* h, const rca_tables* t, const ulm_loc2d* L,
     if (!plane_off) {
         int* poff = (int*)ws_get(h, WS_PLANEOFF, (size_t)(nplanes + 1) * sizeof(int), &st);
         if (!poff) return st;
-        k_list_plane_offsets<<<(nplanes + 1 + 255) / 256, 256, 0, h->stream>>>(L, n2d, cap2d, g.S, nplanes, poff);
+        launch_chain(k_list_plane_offsets, dim3((nplanes + 1 + 255) / 256), dim3(256), 0, h->stream, L, n2d, cap2d, g.S, nplanes, poff);
         plane_off = poff;
     }
     return pair_launch(h, g, L, n2d, cap2d, F, plane_off, best, part, out, cap3d, n3d);
@@ -1179,7 +1187,7 @@ rca_status launch_pair3d_noalloc(rca_handle* h, const rca_tables* t, const ulm_l
     int* best = reinterpret_cast<int*>(base + NA_BEST);
     int* part = reinterpret_cast<int*>(base + NA_PART);
     const int np = (int)nplanes;
-    k_list_plane_offsets<<<(np + 1 + 255) / 256, 256, 0, h->stream>>>(L, n2d, cap2d, g.S, np, poff);
+    launch_chain(k_list_plane_offsets, dim3((np + 1 + 255) / 256), dim3(256), 0, h->stream, L, n2d, cap2d, g.S, np, poff);
     return pair_launch(h, g, L, n2d, cap2d, F, poff, best, part, out, cap3d, n3d);
 }
 
@@ -1200,7 +1208,7 @@ rca_status launch_detect_map(rca_handle* h, const rca_tables* t, const float* ma
     cudaError_t e = cudaFuncSetAttribute(k_detect_map, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_check(h, e, "detect_map smem attribute");
     dim3 grid(nstrip, nplanes);
-    k_detect_map<<<grid, 256, smem, h->stream>>>(map, up, A, M, g.S, g.nz, g.N, score_min, alpha, slots.cand, slots.cnt,
+    launch_chain(k_detect_map, dim3(grid), dim3(256), smem, h->stream, map, up, A, M, g.S, g.nz, g.N, score_min, alpha, slots.cand, slots.cnt,
                                                  slots.part, slots.total, h->d_status);
     if ((st = cuda_check(h, cudaGetLastError(), "detect_map kernel")) != RCA_OK) return st;
     return slots_gather(h, slots, nslots, nstrip, out, cap, n2d, nullptr, nullptr, g);

@@ -43,6 +43,7 @@ __device__ __forceinline__ float2 c_mulc(float2 a, float2 b) { return make_float
 // twiddles w_n^k = exp(-2 pi i k / n), k < n, for n = Xp and then n = Zp
 __global__ void k_mo_twiddles(int xp, int zp, float2* __restrict__ tw)
 {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= xp + zp) return;
     const int n = i < xp ? xp : zp, k = i < xp ? i : i - xp;
@@ -219,6 +220,7 @@ __global__ void __launch_bounds__(32 * ROW_WARPS<T>) k_mo_rows(const float2* __r
                                                  const float2* __restrict__ tw, int frame_base, float2* __restrict__ B,
                                                  float* __restrict__ E)
 {
+    grid_wait();
     constexpr int XP = 16 * T, RW = 32 / T;              // rows per warp
     __shared__ float2 smo[ROW_WARPS<T> * RW * RowBuf<T>::RS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = lane % T, r = lane / T;
@@ -254,6 +256,7 @@ __global__ void __launch_bounds__(T < 16 ? 16 * T : 256, 2) k_mo_cols(float2* __
                                                                       const float2* __restrict__ twz,
                                                                       float4* __restrict__ ref)
 {
+    grid_wait();
     constexpr int ZP = 16 * T, LDZ = T + 2;              // exchange cell (k1, t) in tile row k1 LDZ + t
     extern __shared__ float2 tile[];                     // [16 LDZ][MO_TP]
     const int x0 = blockIdx.x * MO_TILE, k = blockIdx.y;
@@ -304,6 +307,7 @@ __global__ void __launch_bounds__(T < 16 ? 16 * T : 256, 2) k_mo_cols(float2* __
 template <int ZP, bool KEEP>
 __global__ void k_mo_cols_short(float2* __restrict__ B, int nt, int nzs, int xp, float2* __restrict__ ref)
 {
+    grid_wait();
     const int x = threadIdx.x, k = blockIdx.y;
     float2* Bk = B + ((size_t)blockIdx.z * nt + k) * ZP * xp + x;
     float2 v[ZP];
@@ -406,6 +410,7 @@ __global__ void __launch_bounds__(32 * ROW_WARPS<T>) k_mo_peak(const float2* __r
                                                                unsigned* __restrict__ count, float* __restrict__ shifts,
                                                                int* __restrict__ peaks)
 {
+    grid_wait();
     constexpr int XP = 16 * T, RW = 32 / T;
     __shared__ float2 smo[ROW_WARPS<T> * RW * RowBuf<T>::RS];
     __shared__ float s_best[8];
@@ -458,6 +463,7 @@ __global__ void __launch_bounds__(32 * ROW_WARPS<T>) k_mo_peak(const float2* __r
 __global__ void k_mo_combine(const float* __restrict__ shifts, int F, int K, double pitch, double row_m,
                              float* __restrict__ motion)
 {
+    grid_wait();
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
     if (f >= F) return;
     const float* s = shifts + (size_t)f * 2 * K * 3;
@@ -498,11 +504,11 @@ cudaError_t launch_cols(cudaStream_t s, const MotionBufs& b, int nt, int nzs, in
         const int smem = 16 * (T + 2) * MO_TP * (int)sizeof(float2);
         const cudaError_t e = cudaFuncSetAttribute(k_mo_cols<T, KEEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        k_mo_cols<T, KEEP><<<dim3(xp / MO_TILE, nt, nf), T < 16 ? 16 * T : 256, smem, s>>>(b.B, nt, nzs, xp, twz, b.ref);
+        launch_chain(k_mo_cols<T, KEEP>, dim3(xp / MO_TILE, nt, nf), dim3(T < 16 ? 16 * T : 256), smem, s, b.B, nt, nzs, xp, twz, b.ref);
         return cudaGetLastError();
     };
     auto few = [&](auto zc) {
-        k_mo_cols_short<decltype(zc)::value, KEEP><<<dim3(1, nt, nf), xp, 0, s>>>(b.B, nt, nzs, xp, (float2*)b.ref);
+        launch_chain(k_mo_cols_short<decltype(zc)::value, KEEP>, dim3(1, nt, nf), dim3(xp), 0, s, b.B, nt, nzs, xp, (float2*)b.ref);
         return cudaGetLastError();
     };
     switch (logz) {
@@ -524,14 +530,14 @@ cudaError_t run_motion(cudaStream_t s, const MotionBufs& b, const float2* slices
 {
     constexpr int XP = 16 * T, RB = ROW_WARPS<T> * (32 / T);   // rows per k_mo_rows CTA
     const int zp = 1 << logz, npart = (zp + MO_PEAK_ROWS - 1) / MO_PEAK_ROWS;
-    k_mo_twiddles<<<(XP + zp + 255) / 256, 256, 0, s>>>(XP, zp, b.tw);
+    launch_chain(k_mo_twiddles, dim3((XP + zp + 255) / 256), dim3(256), 0, s, XP, zp, b.tw);
     for (int f0 = 0; f0 < F; f0 += chunk) {
         const int nf = std::min(chunk, F - f0);
-        k_mo_rows<T><<<dim3((nzs + RB - 1) / RB, nt, nf), 32 * ROW_WARPS<T>, 0, s>>>(slices, nt, nzs, zp, b.tw, f0, b.B, b.E);
+        launch_chain(k_mo_rows<T>, dim3((nzs + RB - 1) / RB, nt, nf), dim3(32 * ROW_WARPS<T>), 0, s, slices, nt, nzs, zp, b.tw, f0, b.B, b.E);
         cudaError_t e = cudaSuccess;
         if (f0 == 0 && (e = launch_cols<true>(s, b, nt, nzs, XP, logz, 1)) != cudaSuccess) return e;
         if ((e = launch_cols<false>(s, b, nt, nzs, XP, logz, nf)) != cudaSuccess) return e;
-        k_mo_peak<T><<<dim3(npart, nt, nf), 32 * ROW_WARPS<T>, 0, s>>>(b.B, b.E, nt, nzs, zp, b.tw, f0, b.pbest, b.pidx,
+        launch_chain(k_mo_peak<T>, dim3(npart, nt, nf), dim3(32 * ROW_WARPS<T>), 0, s, b.B, b.E, nt, nzs, zp, b.tw, f0, b.pbest, b.pidx,
                                                                        b.count, b.shifts, b.peaks);
     }
     return cudaGetLastError();
@@ -580,6 +586,6 @@ rca_status launch_motion(rca_handle* h, const rca_tables* t, const float2* slice
     default: e = run_motion<16>(h->stream, b, slices, F, nt, nzs, logz, chunk); break;
     }
     if (e != cudaSuccess) return cuda_check(h, e, "motion kernels");
-    k_mo_combine<<<(F + 127) / 128, 128, 0, h->stream>>>(b.shifts, F, g.K, g.pitch, g.dz / g.us, motion);
+    launch_chain(k_mo_combine, dim3((F + 127) / 128), dim3(128), 0, h->stream, b.shifts, F, g.K, g.pitch, g.dz / g.us, motion);
     return cuda_check(h, cudaGetLastError(), "motion kernels");
 }
