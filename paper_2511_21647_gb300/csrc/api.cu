@@ -827,6 +827,8 @@ extern "C" rca_status rca_batch_create(rca_handle* h, int n, const rca_batch_ite
         tmax = std::max(tmax, t->T);
         tmin_all = std::min(tmin_all, t->T);
         if (g.us != 2) b->us2 = false;
+        const S1Layout L1 = stage1_layout(g.N, E.zt, true);
+        if (L1.pair != S1_SPLIT || L1.per != 1 || L1.LW != 1) b->split = false;
         smem = std::max(smem, stage1_smem_bytes(t, E.zt, E.dc, E.ring, esz));
         smem = std::max(smem, stage2_smem_bytes(t, E.zp));
         if (prm) {

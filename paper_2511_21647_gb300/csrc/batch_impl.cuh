@@ -26,7 +26,7 @@ __device__ __forceinline__ int ld_acquire(const int* p)
 }
 
 
-template <typename TS, int MAXR, int TM, int US>
+template <typename TS, int MAXR, int TM, int US, int PAIR>
 __global__ void __launch_bounds__(256, 3) k_batch(const BatchEns* __restrict__ ens, const int4* __restrict__ segs,
                                                  int nseg, int total, int* __restrict__ cnt, int n_counters,
                                                  long long wait_limit, Fir fir, int rf_t, int iq_t, int pt,
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(256, 3) k_batch(const BatchEns* __restrict__ e
             else
                 demod_body<RCA_I16>(a0, a1, a2, xs, E.rf, E.scale, E.mean, E.mix, fir, nt, g.N, g.ns, E.iq, iq_t);
         } else if (stage == BS_STAGE1) {
-            ok = stage1_body<TS, MAXR, false>(a0, a1, a2, smraw, bars, g, E.iq, E.rtab, E.rblk, E.dmax, E.chunks,
+            ok = stage1_body<TS, MAXR, PAIR != S1_UNPAIRED, PAIR>(a0, a1, a2, smraw, bars, g, E.iq, E.rtab, E.rblk, E.dmax, E.chunks,
                                               E.zt, E.dc, E.n_tiles, E.nch, E.ring, E.slices, status);
         } else {
             ok = stage2_body<TM, US>(a0, a1 >> 1, a1 & 1, a2, smraw, &bars[0], g, E.slices, E.sfl, E.sfr, E.lw, E.rot,
@@ -172,10 +172,10 @@ __global__ void __launch_bounds__(256, 3) k_batch(const BatchEns* __restrict__ e
 // ---------------------------------------------------------------------------
 // batched launch
 // ---------------------------------------------------------------------------
-template <typename TS, int MAXR, int TM, int US>
+template <typename TS, int MAXR, int TM, int US, int PAIR>
 static rca_status batch_launch(rca_handle* h, rca_batch* b)
 {
-    auto kern = k_batch<TS, MAXR, TM, US>;
+    auto kern = k_batch<TS, MAXR, TM, US, PAIR>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem);
     if (e != cudaSuccess) return cuda_check(h, e, "batch smem attribute");
     if (b->grid == 0) {
@@ -214,20 +214,23 @@ static rca_status batch_launch(rca_handle* h, rca_batch* b)
     return cuda_check(h, cudaGetLastError(), "batch kernel");
 }
 
-template <typename TS, int MAXR>
+template <typename TS, int MAXR, int PAIR>
 static rca_status batch_tm(rca_handle* h, rca_batch* b)
 {
     // one tap count and two slice rows per plane row in every ensemble: exact,
     // else the generic loop
-    if (b->tmax == 3 && b->tmin_all == 3 && b->us2) return batch_launch<TS, MAXR, 3, 2>(h, b);
-    return batch_launch<TS, MAXR, 0, 0>(h, b);
+    if (b->tmax == 3 && b->tmin_all == 3 && b->us2) return batch_launch<TS, MAXR, 3, 2, PAIR>(h, b);
+    return batch_launch<TS, MAXR, 0, 0, PAIR>(h, b);
 }
 
 template <typename TS>
 static rca_status batch_maxr(rca_handle* h, rca_batch* b)
 {
-    if (b->maxr <= 2) return batch_tm<TS, 2>(h, b);
-    if (b->maxr <= 4) return batch_tm<TS, 4>(h, b);
-    if (b->maxr <= 8) return batch_tm<TS, 8>(h, b);
-    return batch_tm<TS, 16>(h, b);
+    // every ensemble of 32 elements and a row per thread (the tiny geometry's plan):
+    // the split pixel pairs of the standalone kernel
+    if (b->split) return batch_tm<TS, 1, S1_SPLIT>(h, b);
+    if (b->maxr <= 2) return batch_tm<TS, 2, S1_UNPAIRED>(h, b);
+    if (b->maxr <= 4) return batch_tm<TS, 4, S1_UNPAIRED>(h, b);
+    if (b->maxr <= 8) return batch_tm<TS, 8, S1_UNPAIRED>(h, b);
+    return batch_tm<TS, 16, S1_UNPAIRED>(h, b);
 }

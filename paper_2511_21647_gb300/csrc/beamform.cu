@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(256, 4) k_demod(const void* __restrict__ rf, c
     demod_body<RT>(blockIdx.x, blockIdx.y, blockIdx.z, xs, rf, scale, mean, mix, fir, nt, E, ns, iq, iq_t);
 }
 
-template <typename TS, int MAXR, bool PAIR>
+template <typename TS, int MAXR, int PAIR>
 __global__ void __launch_bounds__(256, 2) k_stage1(GeomDev g, const void* __restrict__ iq,
                                                 const unsigned char* __restrict__ rtab, int rblk,
                                                 const int* __restrict__ dmax, const int4* __restrict__ chunks, int zt,
@@ -195,7 +195,7 @@ rca_status launch_ingest(rca_handle* h, const rca_tables* t, const void* rf, rca
     return cuda_check(h, cudaGetLastError(), "ingest kernels");
 }
 
-template <typename TS, int MAXR, bool PAIR>
+template <typename TS, int MAXR, int PAIR>
 static rca_status stage1_launch(rca_handle* h, const rca_tables* t, const void* iq, int F, float2* slices,
                                 int threads)
 {
@@ -221,20 +221,25 @@ static rca_status stage1_dispatch(rca_handle* h, const rca_tables* t, const void
     const int threads = 32 * L.LW * L.RG;
     // the kernel's row loop is exact: every thread owns exactly MAXR rows
     // (or one row, with some warps idle, when the tile has fewer rows than warps)
-    if (!(L.per == 1 || L.per * L.RG == t->s1.zt))
+    if (!(L.per == 1 || L.per * L.slots == t->s1.zt))
         return set_error(h, RCA_ERR_UNSUPPORTED, "Stage-1 row tile %d is not a multiple of %d row groups", t->s1.zt,
-                         L.RG);
-    if (L.pair) {
-        if (L.per == 1) return stage1_launch<TS, 1, true>(h, t, iq, F, slices, threads);
-        if (L.per == 2) return stage1_launch<TS, 2, true>(h, t, iq, F, slices, threads);
-        if (L.per == 4) return stage1_launch<TS, 4, true>(h, t, iq, F, slices, threads);
-        if (L.per == 8) return stage1_launch<TS, 8, true>(h, t, iq, F, slices, threads);
+                         L.slots);
+    if (L.pair == S1_PAIRED) {
+        if (L.per == 1) return stage1_launch<TS, 1, S1_PAIRED>(h, t, iq, F, slices, threads);
+        if (L.per == 2) return stage1_launch<TS, 2, S1_PAIRED>(h, t, iq, F, slices, threads);
+        if (L.per == 4) return stage1_launch<TS, 4, S1_PAIRED>(h, t, iq, F, slices, threads);
+        if (L.per == 8) return stage1_launch<TS, 8, S1_PAIRED>(h, t, iq, F, slices, threads);
+    } else if (L.pair == S1_SPLIT) {
+        if (L.per == 1) return stage1_launch<TS, 1, S1_SPLIT>(h, t, iq, F, slices, threads);
+        if (L.per == 2) return stage1_launch<TS, 2, S1_SPLIT>(h, t, iq, F, slices, threads);
+        if (L.per == 4) return stage1_launch<TS, 4, S1_SPLIT>(h, t, iq, F, slices, threads);
+        if (L.per == 8) return stage1_launch<TS, 8, S1_SPLIT>(h, t, iq, F, slices, threads);
     } else {
-        if (L.per == 1) return stage1_launch<TS, 1, false>(h, t, iq, F, slices, threads);
-        if (L.per == 2) return stage1_launch<TS, 2, false>(h, t, iq, F, slices, threads);
-        if (L.per == 4) return stage1_launch<TS, 4, false>(h, t, iq, F, slices, threads);
-        if (L.per == 8) return stage1_launch<TS, 8, false>(h, t, iq, F, slices, threads);
-        if (L.per == 16) return stage1_launch<TS, 16, false>(h, t, iq, F, slices, threads);
+        if (L.per == 1) return stage1_launch<TS, 1, S1_UNPAIRED>(h, t, iq, F, slices, threads);
+        if (L.per == 2) return stage1_launch<TS, 2, S1_UNPAIRED>(h, t, iq, F, slices, threads);
+        if (L.per == 4) return stage1_launch<TS, 4, S1_UNPAIRED>(h, t, iq, F, slices, threads);
+        if (L.per == 8) return stage1_launch<TS, 8, S1_UNPAIRED>(h, t, iq, F, slices, threads);
+        if (L.per == 16) return stage1_launch<TS, 16, S1_UNPAIRED>(h, t, iq, F, slices, threads);
     }
     return set_error(h, RCA_ERR_UNSUPPORTED, "Stage-1 row tile too tall");
 }

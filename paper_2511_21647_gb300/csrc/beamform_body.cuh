@@ -480,10 +480,11 @@ __device__ __forceinline__ void stage1_range(float (&H)[MAXR][4], float (&G)[MAX
 // Returns false if a bounded wait ran out (the CTA must stop).  The thread
 // owns rows [rg * per, rg * per + per) of the tile, per = ceil(zt / RG)
 // (per <= MAXR; EXACT: per == MAXR and zt == RG * MAXR, or MAXR == 1), and
-// pixel l (plus N - 1 - l when PAIR).
+// pixel l (plus N - 1 - l when paired; PAIR: the S1Layout's pair, whose split form
+// gives the second half of the lanes the next run of rows).
 // rtab: the plan's record table for this arithmetic (FP16 weights for FP16
 // samples, FP32 weights otherwise), one block of rblk bytes per chunk.
-template <typename TS, int MAXR, bool EXACT, bool PAIR = false>
+template <typename TS, int MAXR, bool EXACT, int PAIR = S1_UNPAIRED>
 __device__ __forceinline__ bool stage1_body(int tile, int k, int f, unsigned char* __restrict__ smraw,
                                             uint64_t* bars, const GeomDev& g, const void* __restrict__ iq,
                                             const unsigned char* __restrict__ rtab, int rblk,
@@ -498,14 +499,16 @@ __device__ __forceinline__ bool stage1_body(int tile, int k, int f, unsigned cha
     unsigned char* recs = rng + (size_t)(ring + 1) * RS;      // [2][rblk]
     const int nt = 2 * g.K;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int LW = PAIR ? N >> 6 : (N + 31) >> 5;
+    const int LW = PAIR == S1_PAIRED ? N >> 6 : (PAIR == S1_SPLIT ? N >> 5 : (N + 31) >> 5);
     const int RG = (blockDim.x >> 5) / LW;
     const int lw = warp % LW, rg = warp / LW;
     const int lb = lw * 32;
-    const int l = lb + lane;
+    const int second = PAIR == S1_SPLIT && lb + lane >= N / 2 ? 1 : 0;
+    const int l = lb + lane - second * (N / 2);
     const int m = N - 1 - l;                                   // mirror pixel (PAIR)
-    const int per = (zt + RG - 1) / RG;
-    const int row0 = rg * per;                                 // first tile row of this thread
+    const int slots = PAIR == S1_SPLIT ? 2 * RG : RG;
+    const int per = (zt + slots - 1) / slots;
+    const int row0 = (PAIR == S1_SPLIT ? 2 * rg + second : rg) * per;   // first tile row of this thread
     const int nrow = max(0, min(per, zt - row0));
     const int r0 = tile * zt;
     const int rend = min(r0 + zt, g.nzs);
@@ -516,6 +519,7 @@ __device__ __forceinline__ bool stage1_body(int tile, int k, int f, unsigned cha
     int dmx = 0;
     for (int j = 0; j < nrow; ++j)
         if (r0 + row0 + j < rend) dmx = max(dmx, __ldg(dmax + r0 + row0 + j) + 1);
+    if (PAIR == S1_SPLIT) dmx = __reduce_max_sync(0xffffffffu, dmx);   // both runs of rows in step
 
     if (threadIdx.x == 0) {
         mbar_init(&bars[0], 1);
@@ -585,8 +589,14 @@ __device__ __forceinline__ bool stage1_body(int tile, int k, int f, unsigned cha
     const int Ly = N - 1 - l;
     // warp-uniform range limits: x (e = l - d) for every lane up to xf, for some up to xe;
     // y (e = l + d) for every lane up to yf, for some up to ye
-    const int xf = lb + 31 < N ? lb : -1, xe = min(lb + 31, N - 1);
-    const int yf = N - 32 - lb, ye = N - 1 - lb;
+    int xf = lb + 31 < N ? lb : -1, xe = min(lb + 31, N - 1);
+    int yf = N - 32 - lb, ye = N - 1 - lb;
+    if (PAIR == S1_SPLIT) {
+        xf = __reduce_min_sync(0xffffffffu, l);
+        xe = __reduce_max_sync(0xffffffffu, l);
+        yf = N - 1 - xe;
+        ye = N - 1 - xf;
+    }
     unsigned phase = 0;
     issue(0, 0);
     for (int c = 0; c < nch; ++c) {
@@ -595,7 +605,7 @@ __device__ __forceinline__ bool stage1_body(int tile, int k, int f, unsigned cha
         if (!cta_wait_copies(&bars[b], (phase >> b) & 1u, status)) return false;
         phase ^= 1u << b;
         if (c + 1 < nch) issue(c + 1, b ^ 1);
-        if (cc.w <= cc.z || nrow == 0) continue;
+        if (cc.w <= cc.z || (PAIR != S1_SPLIT && nrow == 0)) continue;
         const unsigned wbase = smem_u32(rng);
         const unsigned rbase = smem_u32(recs + (size_t)b * rblk);
         const unsigned obase = rbase + (unsigned)(zt * dc * 16);
@@ -612,7 +622,7 @@ __device__ __forceinline__ bool stage1_body(int tile, int k, int f, unsigned cha
             if (yf + 1 > d) nx = min(nx, yf + 1);
             if (ye + 1 > d) nx = min(nx, ye + 1);
 #define RCA_S1_RANGE(XM, YM)                                                                                     \
-    stage1_range<TS, MAXR, EXACT, PAIR, XM, YM>(H, G, d, nx, cc.z, zt, l, m, Lx, Ly, row0, nrow, rbase, obase, wbase, \
+    stage1_range<TS, MAXR, EXACT, PAIR != S1_UNPAIRED, XM, YM>(H, G, d, nx, cc.z, zt, l, m, Lx, Ly, row0, nrow, rbase, obase, wbase, \
                                                 RS, dc, (unsigned)((ring - 1) * RS), status)
             switch (xm * 3 + ym) {
             case S1_FULL * 3 + S1_FULL: RCA_S1_RANGE(S1_FULL, S1_FULL); break;
