@@ -226,20 +226,43 @@ __device__ __forceinline__ void demod_body(int bx, int by, int bz, float2* __res
             }
         }
     } else {
-        for (int el = warp; el < DM_NE; el += nwarp) {
-            const int e = e0 + el;
-            const float sc = (rf_t == RCA_I16 && e < E) ? scale[k * E + e] : 1.f;
-            const float* mrow = mean ? mean + ((size_t)k * E + e) * ns : nullptr;
-            for (int sidx = lane; sidx < DM_NT + 30; sidx += 32) {
-                const int n = n0 - 15 + sidx;
-                float2 v = make_float2(0.f, 0.f);
-                if (n >= 0 && n < ns && e < E) {
-                    float x = rf_value(rf, rf_t, (chan0 + e) * ns + n) * sc;
-                    if (mrow) x -= mrow[n];
-                    const float2 m = mix[n];
-                    v = make_float2(x * m.x, x * m.y);
+        // Rows that begin anywhere (ns not a multiple of 4, or buffers off 16 bytes): lanes over samples, single loads.  The
+        // lane's NP mixer values serve all of its warp's elements, and the loads of two elements are issued before any
+        // is used, so 2 NP rows and means are in flight; one load at a time left the kernel waiting for memory (45 frames
+        // of 6 transmissions, 96 elements, 771 FP16 samples: 105 us, 73 now, of which 4 from the short last tile).
+        constexpr int NP = (DM_NT + 30 + 31) / 32;
+        float2 m[NP];
+        bool in[NP];
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const int n = n0 - 15 + lane + 32 * p;
+            in[p] = n >= 0 && n < ns && lane + 32 * p < DM_NT + 30;
+            m[p] = in[p] ? __ldg(mix + n) : make_float2(0.f, 0.f);
+        }
+        for (int el0 = warp; el0 < DM_NE; el0 += 2 * nwarp) {
+            float x[2][NP], mu[2][NP];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int el = el0 + u * nwarp, e = e0 + el;
+                const size_t base = (chan0 + e) * ns + n0 - 15 + lane;
+                const float* mrow = mean ? mean + ((size_t)k * E + e) * ns + n0 - 15 + lane : nullptr;
+#pragma unroll
+                for (int p = 0; p < NP; ++p) {
+                    const bool ok = in[p] && e < E && el < DM_NE;
+                    x[u][p] = ok ? rf_value(rf, rf_t, base + 32 * p) : 0.f;
+                    mu[u][p] = ok && mean ? __ldg(mrow + 32 * p) : 0.f;
                 }
-                xs[el * DM_PITCH + sidx] = v;
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int el = el0 + u * nwarp, e = e0 + el;
+                if (el >= DM_NE) break;
+                const float sc = (rf_t == RCA_I16 && e < E) ? scale[k * E + e] : 1.f;
+#pragma unroll
+                for (int p = 0; p < NP; ++p) {
+                    const float v = x[u][p] * sc - mu[u][p];
+                    if (lane + 32 * p < DM_NT + 30) xs[el * DM_PITCH + lane + 32 * p] = make_float2(v * m[p].x, v * m[p].y);
+                }
             }
         }
     }
@@ -253,6 +276,7 @@ __device__ __forceinline__ void demod_body(int bx, int by, int bz, float2* __res
     const unsigned row = smem_u32(xs + lane * DM_PITCH);
     for (int ob = warp; ob < DM_NT / DM_OB; ob += nwarp) {
         const int s0 = ob * DM_OB;                    // output o sits at window sample o + 15
+        if (n0 + s0 >= ns) break;                     // the record's last tile: no outputs from here on
         uint64_t acc[DM_OB];
 #pragma unroll
         for (int o = 0; o < DM_OB; ++o) acc[o] = 0ull;
