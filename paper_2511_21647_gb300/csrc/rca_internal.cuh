@@ -165,16 +165,19 @@ enum { S1_UNPAIRED = 0, S1_PAIRED = 1, S1_SPLIT = 2 };
 struct S1Layout {
     int LW, RG, slots, per, pair;
 };
-__host__ __device__ inline S1Layout stage1_layout(int N, int zt, bool allow_pair)
+__host__ __device__ constexpr S1Layout stage1_layout(int N, int zt, bool allow_pair)
 {
-    S1Layout s;
+    S1Layout s{};
     if (allow_pair && N % 32 == 0) {
         s.pair = N % 64 == 0 ? S1_PAIRED : S1_SPLIT;
         s.LW = s.pair == S1_PAIRED ? N / 64 : N / 32;
         s.RG = s.LW >= 8 ? 1 : 8 / s.LW;
         s.slots = s.pair == S1_PAIRED ? s.RG : 2 * s.RG;
         s.per = (zt + s.slots - 1) / s.slots;
-        if (s.per <= 8) return s;
+        // the two runs of a split warp go in step through the records, so both have to be whole or both empty: a run past
+        // the tile's rows would read past the record table
+        const bool whole = s.per * s.slots == zt || (s.per == 1 && zt % 2 == 0);
+        if (s.per <= 8 && (s.pair == S1_PAIRED || whole)) return s;
     }
     s.pair = S1_UNPAIRED;
     s.LW = (N + 31) / 32;
@@ -182,6 +185,14 @@ __host__ __device__ inline S1Layout stage1_layout(int N, int zt, bool allow_pair
     s.per = (zt + s.RG - 1) / s.RG;
     return s;
 }
+
+static_assert(stage1_layout(32, 16, true).pair == S1_SPLIT && stage1_layout(32, 8, true).pair == S1_SPLIT &&
+                  stage1_layout(96, 16, true).pair == S1_SPLIT && stage1_layout(128, 1, true).pair == S1_PAIRED,
+              "the plans' row tiles pair");
+static_assert(stage1_layout(32, 1, true).pair == S1_UNPAIRED && stage1_layout(32, 3, true).pair == S1_UNPAIRED &&
+                  stage1_layout(32, 24, true).pair == S1_UNPAIRED && stage1_layout(96, 1, true).pair == S1_UNPAIRED &&
+                  stage1_layout(160, 1, true).pair == S1_UNPAIRED && stage1_layout(224, 3, true).pair == S1_UNPAIRED,
+              "no split warp with one run past the tile");
 
 #define S2_ZP 16       // plane rows per CTA (at most)
 #define S2_THREADS 256
