@@ -226,9 +226,10 @@ static rca_status batch_tm(rca_handle* h, rca_batch* b)
 template <typename TS>
 static rca_status batch_maxr(rca_handle* h, rca_batch* b)
 {
-    // every ensemble of 32 elements and a row per thread (the tiny geometry's plan):
-    // the split pixel pairs of the standalone kernel
-    if (b->split) return batch_tm<TS, 1, S1_SPLIT>(h, b);
+    // every ensemble of 32 elements with row tiles of up to 32 rows (the tiny geometry's default plan and the one its
+    // autotuner picks): the split pixel pairs of the standalone kernel
+    if (b->split == 1) return batch_tm<TS, 1, S1_SPLIT>(h, b);
+    if (b->split == 2) return batch_tm<TS, 2, S1_SPLIT>(h, b);
     if (b->maxr <= 2) return batch_tm<TS, 2, S1_UNPAIRED>(h, b);
     if (b->maxr <= 4) return batch_tm<TS, 4, S1_UNPAIRED>(h, b);
     if (b->maxr <= 8) return batch_tm<TS, 8, S1_UNPAIRED>(h, b);

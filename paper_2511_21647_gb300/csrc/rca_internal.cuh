@@ -587,7 +587,7 @@ struct rca_batch {
     long long wait_limit = RCA_WAIT_CYCLES;
     int maxr = 2, tmax = 1, tmin_all = 1 << 30;
     bool us2 = true;              // every ensemble has two slice rows per plane row
-    bool split = true;            // every ensemble's Stage-1 layout is split with one row per thread
+    int split = 1;                // rows per thread (1, 2) where every ensemble's Stage-1 layout is split, else 0
     size_t smem = 0;
     int grid = 0;
     // launch mode: RCA_BATCH_PERSISTENT (one launch, dependency-ordered queue)

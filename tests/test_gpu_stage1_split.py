@@ -54,3 +54,44 @@ def test_split_stage1(tiny, N, nz, z0, ns, iq_name, tdt, tol):
     got = got[..., 0] + 1j * got[..., 1]
     for rows in (slice(None), slice(-3, None)):                          # and the last rows by themselves; nothing adds up to zero
         assert np.linalg.norm(got[:, :, rows] - ref[:, :, rows]) <= tol * np.linalg.norm(ref[:, :, rows])
+
+
+@pytest.mark.parametrize("tuned", [(False, False), (True, True), (True, False)])
+def test_split_batch_equals_single_calls(tiny, tiny_rf, tuned):
+    """32 elements in a batch with a row per thread (the default tiles), two (the tuned tiles) or both, in each launch mode:
+    the planes of the single calls bit for bit"""
+    from paper_2511_21647_gb300 import _lib as L
+    from paper_2511_21647_gb300 import rca
+    from paper_2511_21647_gb300.pipeline import complex_buffer
+    h = rca.rca_create(0)
+    rca.rca_set_stream(h, torch.cuda.current_stream())
+    g, items, keep = tiny.geom, [], []
+    for tune, F in zip(tuned, (9, 30)):
+        geo = rca.rca_geometry_create(h, g)
+        t = rca.rca_delay_tables(h, geo)
+        rf = tiny_rf.rf[:F].contiguous().cuda()
+        if tune:
+            iq = complex_buffer((F, 2 * len(g.ang_rc), g.ns, g.n_el), L.RCA_C32, "cuda")
+            rca.rca_ingest(h, t, rf, L.RCA_F32, None, F, L.RCA_CLUTTER_MEAN, iq, L.RCA_C32)
+            rca.rca_autotune(h, t, iq, L.RCA_C32, F)
+        items.append(dict(tables=t, rf=rf, n_frames=F, planes=complex_buffer((F, 2, 2, g.n_slab, g.nz, g.n_el), L.RCA_C32, "cuda")))
+        keep.append(geo)
+    ref = []
+    for it in items:
+        p = torch.zeros_like(it["planes"])
+        rca.rca_beamform_projections(h, it["tables"], it["rf"], L.RCA_F32, None, it["n_frames"], rca.bf_params(), p,
+                                     L.RCA_C32)
+        ref.append(p)
+    b = rca.rca_batch_create(h, items, L.RCA_F32, L.RCA_C32, L.RCA_C32)
+    for mode in (L.RCA_BATCH_PERSISTENT, L.RCA_BATCH_STAGED):
+        rca.rca_batch_set_mode(b, mode)
+        for it in items:
+            it["planes"].zero_()
+        rca.rca_batch_run(b, use_graph=False, h=h)
+        assert rca.rca_sync_status(h) == L.RCA_OK
+        assert all(torch.equal(it["planes"], p) for it, p in zip(items, ref))
+    rca.rca_batch_destroy(b)
+    for it, geo in zip(items, keep):
+        rca.rca_tables_destroy(it["tables"])
+        rca.rca_geometry_destroy(geo)
+    rca.rca_destroy(h)
