@@ -231,9 +231,9 @@ def main():
     h, t = sess.h, sess.t
 
     stages = ["ingest", "stage1", "stage2", "enhance", "detect2d", "pair3d"]
-    # kernels per call: mean + demodulation; detect + three scan passes + gather;
-    # list offsets + match + flags + three scan passes + write
-    launches = {"ingest": 2, "stage1": 1, "stage2": 1, "enhance": 1, "detect2d": 5, "pair3d": 7}
+    # kernels per call: mean + demodulation; detect + gather (with its scan);
+    # list offsets + best partners + counts + write
+    launches = {"ingest": 2, "stage1": 1, "stage2": 1, "enhance": 1, "detect2d": 2, "pair3d": 4}
 
     def step(ev=None):
         def mark(i):
@@ -573,6 +573,8 @@ def motion_step(R, L, sess, w, rf_dev, rf_t, scale, iq, iq_t, slices, F, stream,
     R.rca_ingest(sess.h, sess.t, rf_dev, rf_t, scale, F, L.RCA_CLUTTER_NONE, iq, iq_t)
     R.rca_stage1(sess.h, sess.t, iq, iq_t, F, slices)
     motion = torch.zeros((F, 3), device=slices.device)
+    nt, nzs, n_lat = slices.shape[1:4]
+    sl_frame_bytes = nt * (1 << (nzs - 1).bit_length()) * n_lat * 8         # spectra of one frame
 
     def run():
         R.rca_motion_estimate(sess.h, sess.t, slices, F, motion)
@@ -595,7 +597,8 @@ def motion_step(R, L, sess, w, rf_dev, rf_t, scale, iq, iq_t, slices, F, stream,
             "axial_max_error_um": round(1e6 * max(err), 3),
             "lateral_max_um": round(1e6 * float(abs(m[:, :2]).max()), 3),
             "truth": "tissue displacement 0.2 mm sin(2 pi 1 Hz t), t = frame / 400 Hz, axial",
-            "kernels": 5 + 2 * ((F + 63) // 64), "status": R.rca_sync_status(sess.h)}
+            # twiddles, reference columns, combination; rows, columns and peaks of each chunk of 64 MB of spectra
+            "kernels": 3 + 3 * -(-F // max(1, (64 << 20) // sl_frame_bytes)), "status": R.rca_sync_status(sess.h)}
 
 
 def svd_step(R, sess, slices, F, stream, K, rank=16, iters=30):
@@ -1060,13 +1063,14 @@ def learned_form(R, L, sess, planes, F, g, dev, stream, peaks):
             "pairing_ms_per_300_frames": round(split["pair_ms"] * 300 / frames, 3),
             "n2d_per_300_frames": int(split["n2d"] * 300 / frames),
             "cnn_ms_per_300_frames": round(cnn_ms * 300 / frames, 3),
-            "cnn_roofline": {"bound": "tensor", "achieved": round(cnn_gbs, 1), "peak": hbm, "unit": "GB/s",
-                             "frac": round(cnn_gbs / hbm, 4), "bytes_per_pixel": 68,
+            "cnn_roofline": {"bound": "tensor", "achieved": round(tflops, 1), "peak": peak, "unit": "TFLOP/s",
+                             "frac": round(tflops / peak, 4),
+                             "peak_source": "MEASURED_PEAKS.json bf16_tflops (burst)",
                              "kernel": "k_cnn_stream (four layers in one kernel: tcgen05 BF16, TMEM accumulators)",
-                             "peak_source": "MEASURED_PEAKS.json hbm_gbs",
-                             "tensor": {"achieved": round(tflops, 1), "peak": peak, "unit": "TFLOP/s",
-                                        "frac": round(tflops / peak, 4),
-                                        "peak_source": "MEASURED_PEAKS.json bf16_tflops (burst)"}},
+                             "limiter": "shared memory: the tensor cores' operand reads and the layers' rows",
+                             "hbm": {"achieved": round(cnn_gbs, 1), "peak": hbm, "unit": "GB/s",
+                                     "frac": round(cnn_gbs / hbm, 4), "bytes_per_pixel": 68,
+                                     "peak_source": "MEASURED_PEAKS.json hbm_gbs"}},
             "status": R.rca_sync_status(h)}
 
 
