@@ -353,8 +353,7 @@ extern "C" rca_status rca_reserve(rca_handle* h, const rca_geometry* g, int F)
         {WS_A, (size_t)F * 2 * gd.S * gd.nz * gd.N * sizeof(float)},
         {WS_M, (size_t)F * sizeof(float)},
         {WS_CAND, nslots * CAND_CAP * sizeof(ulm_loc2d)},
-        {WS_CANDCNT, nslots * sizeof(int)},
-        {WS_SCAN, (nslots + 1) * sizeof(int)},
+        {WS_CANDCNT, slots_bytes(nslots)},
         {WS_PLANEOFF, ((size_t)F * 2 * gd.S + 1) * sizeof(int)},
     };
     for (auto& w : want)

@@ -150,7 +150,6 @@ __device__ __forceinline__ void split_box(LOAD in, uint64_t (&out)[NB])
 
 // the count of candidate slot s: kept in full, added to the kept total of its
 // chunk of GATHER_SLOTS slots (for the gather's offsets) and to the true total
-#define GATHER_SLOTS 256
 __device__ __forceinline__ void slot_count(int* __restrict__ cnt, int* __restrict__ part,
                                            unsigned long long* __restrict__ total, int s, int n, unsigned* __restrict__ status)
 {
@@ -718,7 +717,8 @@ __global__ void __launch_bounds__(256) k_gather(const ulm_loc2d* __restrict__ ca
         for (int h = GATHER_SLOTS / 2; h > 0; h >>= 1)
             if (off[lo + h] <= dst) lo += h;
         ulm_loc2d e = cand[(size_t)(s0 + lo) * CAND_CAP + (dst - off[lo])];
-        if (A && chk(e.iz >= 0 && e.iz < nz && e.ilat >= 0 && e.ilat < N && e.slab >= 0 && e.slab < S, status))
+        if (A && chk(e.iz >= 0 && e.iz < nz && e.ilat >= 0 && e.ilat < N && e.slab >= 0 && e.slab < S &&
+                         (unsigned)((e.frame * 2 + e.axis) * S + e.slab) < (unsigned)(nslots / nstrip), status))
             e.amp = __ldg(A + (((size_t)(e.frame * 2 + e.axis) * S + e.slab) * nz + e.iz) * N + e.ilat);
         out[dst] = e;
     }
@@ -928,15 +928,15 @@ static rca_status slots_get(rca_handle* h, int nslots, Slots* o)
     rca_status st = RCA_OK;
     o->cand = (ulm_loc2d*)ws_get(h, WS_CAND, (size_t)nslots * CAND_CAP * sizeof(ulm_loc2d), &st);
     if (!o->cand) return st;
-    o->cnt = (int*)ws_get(h, WS_CANDCNT, (size_t)nslots * sizeof(int), &st);
-    if (!o->cnt) return st;
-    // the true total, then the chunks' kept totals
-    const size_t bytes = 16 + (size_t)((nslots + GATHER_SLOTS - 1) / GATHER_SLOTS) * sizeof(int);
-    char* p = (char*)ws_get(h, WS_SCAN, bytes, &st);
+    // the true total, the chunks' kept totals, then the slots' counts.  All are cleared: a block whose wait runs out
+    // counts nothing in the slots that it leaves, and the gather has to find those empty
+    const size_t bytes = slots_bytes(nslots);
+    char* p = (char*)ws_get(h, WS_CANDCNT, bytes, &st);
     if (!p) return st;
     o->total = reinterpret_cast<unsigned long long*>(p);
     o->part = reinterpret_cast<int*>(p + 16);
-    return cuda_check(h, cudaMemsetAsync(p, 0, bytes, h->stream), "candidate totals");
+    o->cnt = o->part + (nslots + GATHER_SLOTS - 1) / GATHER_SLOTS;
+    return cuda_check(h, cudaMemsetAsync(p, 0, bytes, h->stream), "candidate counts");
 }
 
 static rca_status slots_gather(rca_handle* h, const Slots& o, int nslots, int nstrip, ulm_loc2d* out, int cap, int* n2d,

@@ -43,10 +43,9 @@ enum WsSlot {
     WS_A,          // float [F][2][S][nz][N]
     WS_M,          // float [F]
     WS_CAND,       // ulm_loc2d [strips][CAND_CAP]
-    WS_CANDCNT,    // int [strips]
+    WS_CANDCNT,    // candidate totals and counts (slots_bytes)
     WS_PLANEOFF,   // int [planes + 1]
     WS_FLAGS,      // pairing partner of every list entry
-    WS_SCAN,       // totals of the candidate slots
     WS_MISC,       // small scratch
     WS_TRACK,      // tracking: frame offsets, links, flags, positions, per-localisation tracks
     WS_MOTION,     // motion estimation: twiddles, row spectra, reference spectrum, correlations
@@ -232,6 +231,7 @@ void plan_stage2(rca_tables* t, int zp);
 // ---------------------------------------------------------------------------
 #define RCA_MAX_NCC_D 15
 #define CAND_CAP 96       // 2D candidates per (plane, row strip)
+#define GATHER_SLOTS 256  // candidate slots per block of the gather
 #define DET_RS 30         // rows per strip of the heatmap peak search (ulm_detect_map)
 #define NCC_RS 30         // rows per strip of the NCC detection (+ one row above and below: 32 = 8 x 4)
 
@@ -249,6 +249,12 @@ void* ws_get(rca_handle* h, WsSlot slot, size_t bytes, rca_status* st);
 
 // size in bytes of one element of a dtype
 size_t dtype_size(rca_dtype t);
+
+// WS_CANDCNT: the candidates' true total (16 bytes), the kept totals of the gather's chunks, the slots' counts
+inline size_t slots_bytes(size_t nslots)
+{
+    return 16 + ((nslots + GATHER_SLOTS - 1) / GATHER_SLOTS + nslots) * sizeof(int);
+}
 
 // launchers (implemented in the .cu files)
 rca_status launch_tables(rca_handle* h, rca_tables* t);

@@ -1,0 +1,104 @@
+"""The library's host code without a GPU: a stand-in for the CUDA runtime (fake_cudart.c, preloaded into a process of
+its own) records what each call allocates, clears, copies and launches, and runs no kernel."""
+import os
+import shutil
+import subprocess
+import sys
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+SETUP = r"""
+import ctypes as C, math, sys
+from types import SimpleNamespace
+sys.path.insert(0, sys.argv[1])
+from paper_2511_21647_gb300 import _lib as L, rca as R
+def geometry(n_el=32, nz=80, ns=256, P=8, K=1, us=2):
+    return SimpleNamespace(n_el=n_el, P=P, K=K, nz=nz, ns=ns, us=us, pitch=0.2e-3, fc=7.8e6, fs=31.2e6, c=1540.0,
+                           z0=5e-3, dz=0.1e-3, fnum=1.0, ang_rc=[0.05] * K, ang_cr=[-0.05] * K)
+keep = []
+def buf(n):
+    b = C.create_string_buffer(n + 64)
+    keep.append(b)
+    return (C.addressof(b) + 63) // 64 * 64
+def mark(s):
+    R.rca_fp32_probe(h, 0, 1, buf(64))     # a launch of k_fp32_probe in the record
+h = R.rca_create(0)
+"""
+
+
+@pytest.fixture(scope="module")
+def runtime(tmp_path_factory):
+    if not shutil.which("gcc"):
+        pytest.skip("needs gcc")
+    from paper_2511_21647_gb300 import build
+    build()
+    so = str(tmp_path_factory.mktemp("fake") / "libfake_cudart.so")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-O1", "-I/usr/local/cuda/include", os.path.join(HERE, "fake_cudart.c"), "-o", so],
+                   check=True)
+    return so
+
+
+def record(runtime, tmp_path, script, args=""):
+    """the log of `script`, as lists of words"""
+    log = str(tmp_path / "log.txt")
+    env = dict(os.environ, LD_PRELOAD=runtime, FAKE_CUDART_LOG=log, FAKE_CUDART_ARGS=args)
+    r = subprocess.run([sys.executable, "-c", SETUP + script, ROOT], env=env, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-3000:]
+    return [line.split() for line in open(log)]
+
+
+def launch(log, kernel):
+    return next(i for i, w in enumerate(log) if w[0] == "launch" and kernel in w[1])
+
+
+def int32(word):
+    return int(word) & 0xffffffff
+
+
+@pytest.mark.parametrize("call", ["detect2d", "detect_map"])
+def test_candidate_counts_are_cleared_before_detection(runtime, tmp_path, call):
+    """a detection block that gives up writes no count: its slots have to be empty, not what an earlier call left"""
+    script = r"""
+g = R.rca_geometry_create(h, geometry())
+t = R.rca_delay_tables(h, g)
+A, M, out, n = buf(4 * 2 * 4 * 80 * 32 * 4), buf(64), buf(40 * 64), buf(64)
+mark("call")
+""" + (r"""
+R.ulm_detect2d(h, t, A, M, 4, R.make_ulm_params(), out, 64, n)
+""" if call == "detect2d" else r"""
+R.ulm_detect_map(h, t, buf(4 * 2 * 4 * 80 * 32 * 4 * 16), 4, A, M, 4, 0.5, 0.1, out, 64, n)
+""")
+    log = record(runtime, tmp_path, script, "k_gather:5")
+    begin, det = launch(log, "k_fp32_probe"), launch(log, "k_detect")
+    gather = log[launch(log, "k_gather")]
+    cnt, part, total, nslots = int(gather[6]), int(gather[7]), int(gather[8]), int32(gather[9])
+    assert nslots == 4 * 2 * 4 * (3 if call == "detect2d" else 11)
+
+    def cleared(p, n):
+        return any(w[0] == "memset" and int(w[1]) <= p and p + n <= int(w[1]) + int(w[2]) for w in log[begin:det])
+
+    assert cleared(total, 8) and cleared(part, 4 * ((nslots + 255) // 256))
+    assert cleared(cnt, 4 * nslots)
+
+
+def test_reserved_workspace_serves_the_detection(runtime, tmp_path):
+    """after rca_reserve the detection allocates nothing (a capture would refuse it)"""
+    log = record(runtime, tmp_path, r"""
+for nz, F in ((80, 4), (31, 1), (250, 16)):
+    geo = geometry(nz=nz, ns=1100)
+    g = R.rca_geometry_create(h, geo)
+    t = R.rca_delay_tables(h, g)
+    A, M, out, n = buf(F * 2 * 4 * nz * 32 * 4), buf(64), buf(40 * 64), buf(64)
+    R.rca_reserve(h, g, F)
+    mark("call")
+    R.ulm_detect2d(h, t, A, M, F, R.make_ulm_params(), out, 64, n)
+    mark("end")
+""")
+    marks = [i for i, w in enumerate(log) if w[0] == "launch" and "k_fp32_probe" in w[1]]
+    assert len(marks) == 6
+    for a, b in zip(marks[::2], marks[1::2]):
+        assert [w for w in log[a:b] if w[0] == "launch" and "k_gather" in w[1]]
+        assert not [w for w in log[a:b] if w[0] == "malloc"]
