@@ -172,7 +172,8 @@ __device__ __forceinline__ void demod_body(int bx, int by, int bz, float2* __res
     const int k = fk % nt;
     const size_t chan0 = (size_t)fk * E;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    // stage (rf - mean) * exp(-j 2 pi fc t_n) for samples n0-15 .. n0+DM_NT+14
+    // stage (rf - mean) * exp(-j 2 pi fc t_n) for samples n0-15 .. n0+DM_NT+14.  The mean is read with __ldcg: in the
+    // persistent batch other blocks of the same launch write it, which the read-only path (__ldg) must not be used for
     const bool quads = (ns & 3) == 0 && (reinterpret_cast<uintptr_t>(rf) & 15) == 0 &&
                        (reinterpret_cast<uintptr_t>(mean) & 15) == 0;
     if (quads) {
@@ -201,7 +202,7 @@ __device__ __forceinline__ void demod_body(int bx, int by, int bz, float2* __res
                 r[u] = mu[u] = ma[u] = mb[u] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (idx < ITEMS && nb >= 0 && nb < ns && e < E) {
                     r[u] = rf_quad<RT>(rf, (chan0 + e) * ns + nb);
-                    if (mean) mu[u] = __ldg(reinterpret_cast<const float4*>(mean + ((size_t)k * E + e) * ns + nb));
+                    if (mean) mu[u] = __ldcg(reinterpret_cast<const float4*>(mean + ((size_t)k * E + e) * ns + nb));
                     ma[u] = __ldg(reinterpret_cast<const float4*>(mix + nb));
                     mb[u] = __ldg(reinterpret_cast<const float4*>(mix + nb + 2));
                 }
@@ -250,7 +251,7 @@ __device__ __forceinline__ void demod_body(int bx, int by, int bz, float2* __res
                 for (int p = 0; p < NP; ++p) {
                     const bool ok = in[p] && e < E && el < DM_NE;
                     x[u][p] = ok ? rf_value(rf, rf_t, base + 32 * p) : 0.f;
-                    mu[u][p] = ok && mean ? __ldg(mrow + 32 * p) : 0.f;
+                    mu[u][p] = ok && mean ? __ldcg(mrow + 32 * p) : 0.f;
                 }
             }
 #pragma unroll
