@@ -287,7 +287,10 @@ rca_status ulm_enhance(rca_handle* h, const rca_tables* t, const void* planes, r
  * sub-pixel 3x3 regional peaks with NCC >= ncc_min and A >= alpha M_t (ties
  * to the earlier raster pixel), parabolic sub-pixel refinement.
  *   out: capacity cap2d; *n2d_dev (device int) receives the true count even
- *   when it exceeds cap2d (then the status word gets CAPACITY).
+ *   when it exceeds cap2d (then the status word gets CAPACITY).  A strip of 30
+ *   rows of one plane keeps its first 96 entries; where more were found the
+ *   status word gets CAPACITY too, and the entries between those kept and the
+ *   count have frame = n_frames (they sort last and pair with nothing).
  *   ncc_out: optional [F][2][S][nz][N] float copy of the NCC maps (NULL = none).
  *   plane_offsets: optional device int [F*2*S + 1] list offset of each plane. */
 rca_status ulm_detect2d(rca_handle* h, const rca_tables* t, const float* A, const float* M,

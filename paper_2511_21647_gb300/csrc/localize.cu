@@ -2,6 +2,7 @@
 // XZ / YZ pairing (Sec. II-A4, Fig. 1e, Fig. 1g).
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <mutex>
 
 #include "rca_internal.cuh"
@@ -149,7 +150,8 @@ __device__ __forceinline__ void split_box(LOAD in, uint64_t (&out)[NB])
 }
 
 // the count of candidate slot s: kept in full, added to the kept total of its
-// chunk of GATHER_SLOTS slots (for the gather's offsets) and to the true total
+// chunk of GATHER_SLOTS slots (for the gather's offsets), to the true total and,
+// what does not fit the slot, to the dropped total (total[1])
 __device__ __forceinline__ void slot_count(int* __restrict__ cnt, int* __restrict__ part,
                                            unsigned long long* __restrict__ total, int s, int n, unsigned* __restrict__ status)
 {
@@ -158,7 +160,10 @@ __device__ __forceinline__ void slot_count(int* __restrict__ cnt, int* __restric
         atomicAdd(part + s / GATHER_SLOTS, min(n, CAND_CAP));
         atomicAdd(total, (unsigned long long)n);
     }
-    if (n > CAND_CAP) atomicOr(status, ST_CAPACITY);
+    if (n > CAND_CAP) {
+        atomicAdd(total + 1, (unsigned long long)(n - CAND_CAP));
+        atomicOr(status, ST_CAPACITY);
+    }
 }
 
 // Whether NCC row ro, column l of the NCC rows sN is a 3 x 3 regional maximum.
@@ -683,7 +688,11 @@ __device__ __forceinline__ int block_offset(const int* __restrict__ part, int n,
 // the chunk's entries are spread over its threads.  A non-null: each entry's
 // amplitude is read here from A [plane][nz][N] at its pixel (the detection kernel
 // leaves it to this highly parallel pass).  poff (optional): the list offset of
-// every plane, of nstrip slots each.
+// every plane, of nstrip slots each.  Where slots dropped candidates, the count
+// goes past the entries kept; what it covers beyond them becomes entries of frame F,
+// which sort last and pair with nothing, so that a list is in order over its count
+// (with whatever the buffer held there, the pairing's plane offsets were wrong and
+// its searches ran over the whole list: 58 ms instead of 0.58 for a count of 1.3 million, 0.49 of them kept).
 __global__ void __launch_bounds__(256) k_gather(const ulm_loc2d* __restrict__ cand, const int* __restrict__ cnt,
                                                 const int* __restrict__ part, const unsigned long long* __restrict__ total,
                                                 int nslots, int nstrip, ulm_loc2d* __restrict__ out, int cap,
@@ -704,6 +713,15 @@ __global__ void __launch_bounds__(256) k_gather(const ulm_loc2d* __restrict__ ca
         if (s == nslots - 1) poff[nslots / nstrip] = at + own;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) *n_out = (int)min(*total, 0x7fffffffull);
+    if (total[1] != 0) {
+        // word by word: entry by entry (40 bytes a lane) took ten times as long
+        constexpr int EW = sizeof(ulm_loc2d) / 4;
+        const int F = nslots / nstrip / (2 * S);
+        int* w = reinterpret_cast<int*>(out);
+        const long long end = (long long)min(*total, (unsigned long long)cap) * EW;
+        for (long long i = (long long)(*total - total[1]) * EW + blockIdx.x * 256 + threadIdx.x; i < end; i += 256 * gridDim.x)
+            w[i] = i % EW == offsetof(ulm_loc2d, frame) / 4 ? F : 0;
+    }
     __syncthreads();
     const int base = off[0], n = all - base;
     for (int i = threadIdx.x; i < n; i += 256) {
