@@ -870,12 +870,17 @@ extern "C" rca_status ulm_cnn_forward(ulm_cnn* c, const float* A, const float* M
     if (!A || !heat) return set_error(c->h, RCA_ERR_INVALID_ARG, "null input or heatmap");
     rca_status st = cnn_check_shape(c, B, H, W);
     if (st != RCA_OK) return st;
-    // the kernel stores 16-byte vectors; a heatmap at another alignment is copied out of the network's own
-    float* direct = (reinterpret_cast<uintptr_t>(heat) & 15) == 0 ? heat : c->heat;
+    // the kernel stores 16-byte vectors, and stores while other blocks still read: a heatmap at another alignment, or over
+    // the memory of the input or its maxima, is copied out of the network's own
+    const size_t px = (size_t)B * H * W, nM = M ? ((size_t)B + std::max(ppf, 1) - 1) / std::max(ppf, 1) : 0;
+    auto over = [&](const float* p, size_t n) {
+        const uintptr_t a = reinterpret_cast<uintptr_t>(heat), b = reinterpret_cast<uintptr_t>(p);
+        return a < b + n * 4 && b < a + px * CNN_UP * CNN_UP * 4;
+    };
+    float* direct = (reinterpret_cast<uintptr_t>(heat) & 15) == 0 && !over(A, px) && !over(M, nM) ? heat : c->heat;
     if ((st = cnn_forward<false>(c, A, M, ppf, B, H, W, direct)) != RCA_OK || direct == heat) return st;
     return cuda_check(c->h,
-                      cudaMemcpyAsync(heat, c->heat, (size_t)B * H * W * CNN_UP * CNN_UP * 4, cudaMemcpyDeviceToDevice,
-                                      c->h->stream),
+                      cudaMemcpyAsync(heat, c->heat, px * CNN_UP * CNN_UP * 4, cudaMemcpyDeviceToDevice, c->h->stream),
                       "heatmap copy");
 }
 

@@ -692,7 +692,7 @@ __device__ __forceinline__ int block_offset(const int* __restrict__ part, int n,
 // goes past the entries kept; what it covers beyond them becomes entries of frame F,
 // which sort last and pair with nothing, so that a list is in order over its count
 // (with whatever the buffer held there, the pairing's plane offsets were wrong and
-// its searches ran over the whole list: 58 ms instead of 0.58 for a count of 1.3 million, 0.49 of them kept).
+// its searches ran over the whole list: 58 ms instead of 0.58 for a count of 1.31 million, 0.49 million kept).
 __global__ void __launch_bounds__(256) k_gather(const ulm_loc2d* __restrict__ cand, const int* __restrict__ cnt,
                                                 const int* __restrict__ part, const unsigned long long* __restrict__ total,
                                                 int nslots, int nstrip, ulm_loc2d* __restrict__ out, int cap,

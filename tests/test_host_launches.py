@@ -102,3 +102,23 @@ for nz, F in ((80, 4), (31, 1), (250, 16)):
     for a, b in zip(marks[::2], marks[1::2]):
         assert [w for w in log[a:b] if w[0] == "launch" and "k_gather" in w[1]]
         assert not [w for w in log[a:b] if w[0] == "malloc"]
+
+
+def test_inference_over_its_input_goes_through_the_own_heatmap(runtime, tmp_path):
+    """a heatmap over the memory of the input planes or of their maxima is not stored while others are read"""
+    log = record(runtime, tmp_path, r"""
+B, H, W = 6, 20, 32
+px = B * H * W
+net = R.ulm_cnn_create(h, max_pixels=px)
+mem = buf(4 * 40 * px)
+ends = 4 * 16 * px
+for A, M, heat in ((mem, 0, mem), (mem + 64, 0, mem), (mem + ends - 4, 0, mem), (mem, 0, mem + 4 * px - 16), (mem + ends, mem + 64, mem),
+                   (mem + ends + 64, mem + ends - 4, mem),
+                   (mem + ends, 0, mem), (mem, 0, mem + 4 * px), (mem + ends, mem + ends + 4 * px, mem), (mem, mem + 4 * px, mem + 4 * px + 16)):
+    mark("call")
+    R.ulm_cnn_infer(net, A, M or None, 2, B, H, W, heat)
+mark("end")
+""")
+    marks = [i for i, w in enumerate(log) if w[0] == "launch" and "k_fp32_probe" in w[1]]
+    copied = [any(w[0] == "memcpy" for w in log[a:b]) for a, b in zip(marks, marks[1:])]
+    assert copied == [True] * 6 + [False] * 4
