@@ -452,8 +452,9 @@ __global__ void __launch_bounds__(SV_THREADS) k_svd_orth(float2* __restrict__ Yg
 
 // ---------------------------------------------------------------------------
 // The whole orthogonal iteration of one transmission in one cluster of eight
-// CTAs.  Each CTA holds an eighth of the rows of C_k (in shared memory where it
-// fits) and the whole basis V; a step is
+// CTAs.  Each CTA owns an eighth of the rows of C_k (up to 320 frames, ten rows per
+// lane, they fit its shared memory; beyond, each step reads them from L2) and holds
+// the whole basis V; a step is
 //   product   the CTA's rows of C V, one row and three columns per thread
 //   exchange  its rows to every CTA's V (distributed shared memory), between two
 //             cluster barriers: V is read by the product until the first
@@ -466,6 +467,7 @@ __global__ void __launch_bounds__(SV_THREADS) k_svd_orth(float2* __restrict__ Yg
 // ---------------------------------------------------------------------------
 #define SVI_CTAS 8
 #define SVI_FMAX 512                                   // 32 lanes x 16 rows of a column
+#define SVI_FSMEM 320                                  // C's rows in shared memory up to here (10 rows of a column)
 
 __device__ __forceinline__ void svi_cluster_sync()
 {
@@ -486,7 +488,7 @@ inline SviSmem svi_smem(int F, int nb)
     s.v = 0;
     s.part = s.v + F * s.ld * 8;
     s.c = s.part + s.rows * nb * 8;
-    s.c_in = (size_t)s.c + (size_t)s.rows * s.ldc * 8 <= 224 * 1024;
+    s.c_in = F <= SVI_FSMEM;                           // 197 KB at most (33 columns)
     s.bytes = s.c + (s.c_in ? s.rows * s.ldc * 8 : 0);
     return s;
 }
@@ -856,8 +858,8 @@ rca_status launch_clutter_svd(rca_handle* h, const rca_tables* t, float2* slices
     // the cluster kernel keeps a column in a warp's registers, 16 rows per lane at most
     if (F <= SVI_FMAX) {
         const SviSmem L = svi_smem(F, nb);
-        auto kern = F <= 320 && L.c_in ? (nb <= 32 ? k_svd_iterate<10, 2, true> : k_svd_iterate<10, 3, true>)
-                                       : (nb <= 32 ? k_svd_iterate<16, 2, false> : k_svd_iterate<16, 3, false>);
+        auto kern = L.c_in ? (nb <= 32 ? k_svd_iterate<10, 2, true> : k_svd_iterate<10, 3, true>)
+                           : (nb <= 32 ? k_svd_iterate<16, 2, false> : k_svd_iterate<16, 3, false>);
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L.bytes);
         if (e != cudaSuccess) return cuda_check(h, e, "subspace smem attribute");
         kern<<<dim3(SVI_CTAS, nt), SV_THREADS, L.bytes, h->stream>>>(C, F, nb, iters, L, Q);

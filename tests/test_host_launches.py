@@ -122,3 +122,20 @@ mark("end")
     marks = [i for i, w in enumerate(log) if w[0] == "launch" and "k_fp32_probe" in w[1]]
     copied = [any(w[0] == "memcpy" for w in log[a:b]) for a, b in zip(marks, marks[1:])]
     assert copied == [True] * 6 + [False] * 4
+
+
+def test_iteration_asks_for_the_shared_memory_it_uses(runtime, tmp_path):
+    """the subspace iteration's basis and products, and C's rows only for the kernels that keep them there"""
+    sizes = [(9, 3), (300, 16), (320, 32), (321, 16), (360, 30), (400, 4), (512, 16), (512, 22)]
+    log = record(runtime, tmp_path, rf"""
+g = R.rca_geometry_create(h, geometry(nz=4))
+t = R.rca_delay_tables(h, g)
+for F, rank in {sizes}:
+    R.rca_clutter_svd(h, t, buf(F * 2 * 7 * 32 * 8), F, rank)
+""")
+    found = [w for w in log if w[0] == "launch" and "k_svd_iterate" in w[1]]
+    assert len(found) == len(sizes)
+    for (F, rank), w in zip(sizes, found):
+        nb, rows, in_smem = rank + 1, -(-F // 8), "Lb1E" in w[1]
+        assert int(w[4]) == 8 * (F * (nb | 1) + rows * nb + (rows * (F | 1) if in_smem else 0)), (F, rank)
+        assert in_smem == (F <= 320) and int(w[4]) <= 227 * 1024 - 1024
