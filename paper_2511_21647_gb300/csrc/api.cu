@@ -829,7 +829,7 @@ extern "C" rca_status rca_batch_create(rca_handle* h, int n, const rca_batch_ite
         const S1Layout L1 = stage1_layout(g.N, E.zt, true);
         // the kernel's row loop is exact: one row count for the whole batch (a mixed batch stays unpaired)
         if (e == 0) b->split = L1.per;
-        if (L1.pair != S1_SPLIT || L1.LW != 1 || L1.per > 2 || L1.per != b->split) b->split = 0;
+        if (L1.pair != S1_SPLIT || L1.LW != 1 || L1.per > 2 || L1.per != b->split || !stage1_exact(L1, E.zt)) b->split = 0;
         smem = std::max(smem, stage1_smem_bytes(t, E.zt, E.dc, E.ring, esz));
         smem = std::max(smem, stage2_smem_bytes(t, E.zp));
         if (prm) {

@@ -221,7 +221,7 @@ static rca_status stage1_dispatch(rca_handle* h, const rca_tables* t, const void
     const int threads = 32 * L.LW * L.RG;
     // the kernel's row loop is exact: every thread owns exactly MAXR rows
     // (or one row, with some warps idle, when the tile has fewer rows than warps)
-    if (!(L.per == 1 || L.per * L.slots == t->s1.zt))
+    if (!stage1_exact(L, t->s1.zt))
         return set_error(h, RCA_ERR_UNSUPPORTED, "Stage-1 row tile %d is not a multiple of %d row groups", t->s1.zt,
                          L.slots);
     if (L.pair == S1_PAIRED) {

@@ -503,10 +503,10 @@ __device__ __forceinline__ void stage1_range(float (&H)[MAXR][4], float (&G)[MAX
 }
 
 // Returns false if a bounded wait ran out (the CTA must stop).  The thread
-// owns rows [rg * per, rg * per + per) of the tile, per = ceil(zt / RG)
-// (per <= MAXR; EXACT: per == MAXR and zt == RG * MAXR, or MAXR == 1), and
-// pixel l (plus N - 1 - l when paired; PAIR: the S1Layout's pair, whose split form
-// gives the second half of the lanes the next run of rows).
+// owns a run of per = ceil(zt / slots) rows of the tile (S1Layout; per <= MAXR;
+// EXACT: per == MAXR and stage1_exact, which the host checks), and pixel l (plus
+// N - 1 - l when paired; PAIR: the layout's pair, whose split form gives the second
+// half of the lanes the next run of rows).
 // rtab: the plan's record table for this arithmetic (FP16 weights for FP16
 // samples, FP32 weights otherwise), one block of rblk bytes per chunk.
 template <typename TS, int MAXR, bool EXACT, int PAIR = S1_UNPAIRED>

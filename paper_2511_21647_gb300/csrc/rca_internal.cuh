@@ -164,6 +164,14 @@ enum { S1_UNPAIRED = 0, S1_PAIRED = 1, S1_SPLIT = 2 };
 struct S1Layout {
     int LW, RG, slots, per, pair;
 };
+// What the kernels' exact row loops need of a tile of zt rows: whole runs, or one row
+// a thread with the last runs empty.  The two runs of a split warp go in step through
+// the records, so there both are whole or both empty: a run past the tile's rows would
+// read past the record table.
+__host__ __device__ constexpr bool stage1_exact(const S1Layout& s, int zt)
+{
+    return s.per * s.slots == zt || (s.per == 1 && (s.pair != S1_SPLIT || zt % 2 == 0));
+}
 __host__ __device__ constexpr S1Layout stage1_layout(int N, int zt, bool allow_pair)
 {
     S1Layout s{};
@@ -173,10 +181,7 @@ __host__ __device__ constexpr S1Layout stage1_layout(int N, int zt, bool allow_p
         s.RG = s.LW >= 8 ? 1 : 8 / s.LW;
         s.slots = s.pair == S1_PAIRED ? s.RG : 2 * s.RG;
         s.per = (zt + s.slots - 1) / s.slots;
-        // the two runs of a split warp go in step through the records, so both have to be whole or both empty: a run past
-        // the tile's rows would read past the record table
-        const bool whole = s.per * s.slots == zt || (s.per == 1 && zt % 2 == 0);
-        if (s.per <= 8 && (s.pair == S1_PAIRED || whole)) return s;
+        if (s.per <= 8 && (s.pair == S1_PAIRED || stage1_exact(s, zt))) return s;
     }
     s.pair = S1_UNPAIRED;
     s.LW = (N + 31) / 32;

@@ -1,6 +1,7 @@
 """The library's host code without a GPU: a stand-in for the CUDA runtime (fake_cudart.c, preloaded into a process of
 its own) records what each call allocates, clears, copies and launches, and runs no kernel."""
 import os
+import re
 import shutil
 import subprocess
 import sys
@@ -139,3 +140,25 @@ for F, rank in {sizes}:
         nb, rows, in_smem = rank + 1, -(-F // 8), "Lb1E" in w[1]
         assert int(w[4]) == 8 * (F * (nb | 1) + rows * nb + (rows * (F | 1) if in_smem else 0)), (F, rank)
         assert in_smem == (F <= 320) and int(w[4]) <= 227 * 1024 - 1024
+
+
+@pytest.mark.parametrize("widths,form", [((32,), (1, 2)), ((32, 32), (1, 2)), ((32, 64), (4, 0)), ((36,), (4, 0)), ((64,), (4, 0)),
+                                         ((96,), (8, 0)), ((96, 32), (8, 0)), ((128, 32), (8, 0))])
+def test_batch_row_loop_fits_its_tiles(runtime, tmp_path, widths, form):
+    """rows per thread and pixel pairing of the batch kernel: the exact split form only where every ensemble's tiles have
+    whole runs for it, else the loop with the tallest ensemble's rows per thread (tiles of 16 rows)"""
+    log = record(runtime, tmp_path, rf"""
+items = []
+for n_el in {widths}:
+    g = R.rca_geometry_create(h, geometry(n_el=n_el, P=4))
+    t = R.rca_delay_tables(h, g)
+    items.append(dict(tables=t, rf=buf(3 * 2 * n_el * 256 * 4), n_frames=3, planes=buf(3 * 4 * n_el // 4 * 80 * n_el * 8)))
+b = R.rca_batch_create(h, items, L.RCA_F32, L.RCA_C32, L.RCA_C32)
+R.rca_batch_set_mode(b, L.RCA_BATCH_STAGED)
+R.rca_batch_run(b, False, h)
+""")
+    names = [w[1] for w in log if w[0] == "launch" and "k_batch" in w[1]]
+    assert len(names) == 4
+    for name in names:
+        maxr, _, _, pair = (int(x) for x in re.findall(r"Li(\d+)E", name))
+        assert (maxr, pair) == form
