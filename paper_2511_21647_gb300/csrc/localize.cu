@@ -685,9 +685,10 @@ __device__ __forceinline__ int block_offset(const int* __restrict__ part, int n,
 // Copy the kept candidates of a chunk of slots to their place in the output list:
 // the chunk's offset is the sum of the totals before it, a slot's a scan of the
 // counts in the block (one launch instead of three scan kernels and a gather), and
-// the chunk's entries are spread over its threads.  A non-null: each entry's
-// amplitude is read here from A [plane][nz][N] at its pixel (the detection kernel
-// leaves it to this highly parallel pass).  poff (optional): the list offset of
+// the chunk's entries are spread over the threads of gridDim.y blocks, which scan
+// alike (slots_gather's rule).  A non-null: each entry's amplitude is read here from
+// A [plane][nz][N] at its pixel (the detection kernel leaves it to this highly
+// parallel pass).  poff (optional): the list offset of
 // every plane, of nstrip slots each.  Where slots dropped candidates, the count
 // goes past the entries kept; what it covers beyond them becomes entries of frame F,
 // which sort last and pair with nothing, so that a list is in order over its count
@@ -708,23 +709,24 @@ __global__ void __launch_bounds__(256) k_gather(const ulm_loc2d* __restrict__ ca
     const int at = block_offset(part, blockIdx.x, own, red, &all);
     off[threadIdx.x] = at;
     if (threadIdx.x == 0) off[GATHER_SLOTS] = all;
-    if (poff) {
+    if (poff && blockIdx.y == 0) {
         if (s < nslots && s % nstrip == 0) poff[s / nstrip] = at;
         if (s == nslots - 1) poff[nslots / nstrip] = at + own;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) *n_out = (int)min(*total, 0x7fffffffull);
+    const int turn = 256 * gridDim.y, first = 256 * blockIdx.y + threadIdx.x;
+    if (blockIdx.x == 0 && first == 0) *n_out = (int)min(*total, 0x7fffffffull);
     if (total[1] != 0) {
         // word by word: entry by entry (40 bytes a lane) took ten times as long
         constexpr int EW = sizeof(ulm_loc2d) / 4;
         const int F = nslots / nstrip / (2 * S);
         int* w = reinterpret_cast<int*>(out);
         const long long end = (long long)min(*total, (unsigned long long)cap) * EW;
-        for (long long i = (long long)(*total - total[1]) * EW + blockIdx.x * 256 + threadIdx.x; i < end; i += 256 * gridDim.x)
+        for (long long i = (long long)(*total - total[1]) * EW + blockIdx.x * turn + first; i < end; i += turn * gridDim.x)
             w[i] = i % EW == offsetof(ulm_loc2d, frame) / 4 ? F : 0;
     }
     __syncthreads();
     const int base = off[0], n = all - base;
-    for (int i = threadIdx.x; i < n; i += 256) {
+    for (int i = first; i < n; i += turn) {
         const int dst = base + i;
         if (dst >= cap) {
             atomicOr(status, ST_CAPACITY);
@@ -961,7 +963,14 @@ static rca_status slots_gather(rca_handle* h, const Slots& o, int nslots, int ns
                                int* poff, const float* A, const GeomDev& g)
 {
     if (nslots > SCAN_MAX) return set_error(h, RCA_ERR_UNSUPPORTED, "scan over more than %d entries", SCAN_MAX);
-    launch_chain(k_gather, dim3((nslots + GATHER_SLOTS - 1) / GATHER_SLOTS), dim3(256), 0, h->stream, 
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // up to eight blocks a chunk, as long as there are no more than four per SM: with one, 20 frames of 250 x 128
+    // planes have 23 blocks, which took 70 us for the 150 000 entries of 26 a slot (detection 162 us, now 104)
+    const int chunks = (nslots + GATHER_SLOTS - 1) / GATHER_SLOTS;
+    const int ny = std::max(1, std::min(8, 4 * sms / chunks));
+    launch_chain(k_gather, dim3(chunks, ny), dim3(256), 0, h->stream,
         o.cand, o.cnt, o.part, o.total, nslots, nstrip, out, cap, n2d, poff, A, g.S, g.nz, g.N, h->d_status);
     return cuda_check(h, cudaGetLastError(), "gather kernel");
 }

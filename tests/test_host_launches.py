@@ -162,3 +162,16 @@ R.rca_batch_run(b, False, h)
     for name in names:
         maxr, _, _, pair = (int(x) for x in re.findall(r"Li(\d+)E", name))
         assert (maxr, pair) == form
+
+
+def test_gather_spreads_few_chunks_of_slots(runtime, tmp_path):
+    """chunks of 256 candidate slots: up to eight blocks each while they are few, one for a long ensemble"""
+    log = record(runtime, tmp_path, r"""
+g = R.rca_geometry_create(h, geometry())
+t = R.rca_delay_tables(h, g)
+out, n = buf(40 * 64), buf(64)
+for F in (1, 64, 300, 1700, 3000):
+    R.ulm_detect2d(h, t, buf(64), buf(64), F, R.make_ulm_params(), out, 64, n)
+""")
+    grids = [tuple(int(x) for x in w[2].split(",")) for w in log if w[0] == "launch" and "k_gather" in w[1]]
+    assert grids == [(1, 8, 1), (6, 8, 1), (29, 8, 1), (160, 3, 1), (282, 2, 1)]
