@@ -807,64 +807,86 @@ __device__ __forceinline__ bool pair_better(float a, int p, float pa, int q, flo
     return c64 < d64 || (c64 == d64 && p < q);
 }
 
-// Every entry's partner on the other axis: the eligible entry of the least cost in
-// the plane of its own slab's counterpart, ties to the lower index (-1: none).  A
-// pair is a match when each is the other's partner.  Eight lanes share an entry (a
-// plane holds a few to a few tens of entries; one thread per XZ entry that searched
-// there and back took 222 us on the paper's list and 25 us on a tiny one, a serial
-// chain of loads and FP64 divisions; now 70 and 5).
-#define PAIR_LANES 8
-__global__ void __launch_bounds__(256) k_pair_best(const ulm_loc2d* __restrict__ L, const int* __restrict__ n2d, int cap2d,
-                                                   int F, int S, int P, const int* __restrict__ poff, int* __restrict__ best)
+// The partner of entry e: the eligible entry of the least cost in the plane of its
+// slab's counterpart on the other axis, ties to the lower index (0x7fffffff: none, or
+// !act).  LANES consecutive lanes share an entry.
+template <int LANES>
+__device__ __forceinline__ int pair_search(const ulm_loc2d* __restrict__ L, int n, const ulm_loc2d& e, bool act, int F, int S,
+                                           int P, const int* __restrict__ poff)
 {
-    grid_wait();
-    const int n = min(*n2d, cap2d), sub = threadIdx.x % PAIR_LANES;
-    constexpr int PER = 256 / PAIR_LANES;
-    for (int a0 = blockIdx.x * PER; a0 < n; a0 += gridDim.x * PER) {
-        const int a = a0 + threadIdx.x / PAIR_LANES;
-        int b = 0x7fffffff;
-        float amp = 0.f, pa = 0.f;
-        if (a < n) {
-            const ulm_loc2d x = L[a];
-            amp = x.amp;
-            const int slab = x.ilat / P;
-            if ((unsigned)x.axis < 2u && x.frame >= 0 && x.frame < F && x.ilat >= 0 && slab < S) {
-                const int pl = (x.frame * 2 + 1 - x.axis) * S + slab;
-                const int q1 = min(poff[pl + 1], n);
-                for (int q = poff[pl] + sub; q < q1; q += PAIR_LANES) {
-                    const ulm_loc2d y = L[q];
-                    if ((x.axis == 0 ? pair_ok(x, y, P) : pair_ok(y, x, P)) &&
-                        (b == 0x7fffffff || pair_better(amp, q, y.amp, b, pa))) {
-                        b = q;
-                        pa = y.amp;
-                    }
-                }
+    int b = 0x7fffffff;
+    float pa = 0.f;
+    const int slab = e.ilat / P;
+    if (act && (unsigned)e.axis < 2u && e.frame >= 0 && e.frame < F && e.ilat >= 0 && slab < S) {
+        const int pl = (e.frame * 2 + 1 - e.axis) * S + slab;
+        const int q1 = min(poff[pl + 1], n);
+        for (int q = poff[pl] + (int)(threadIdx.x % LANES); q < q1; q += LANES) {
+            const ulm_loc2d y = L[q];
+            if ((e.axis == 0 ? pair_ok(e, y, P) : pair_ok(y, e, P)) &&
+                (b == 0x7fffffff || pair_better(e.amp, q, y.amp, b, pa))) {
+                b = q;
+                pa = y.amp;
             }
         }
+    }
 #pragma unroll
-        for (int o = PAIR_LANES / 2; o > 0; o >>= 1) {
-            const int ob = __shfl_xor_sync(0xffffffffu, b, o);
-            const float oa = __shfl_xor_sync(0xffffffffu, pa, o);
-            if (ob != 0x7fffffff && (b == 0x7fffffff || pair_better(amp, ob, oa, b, pa))) {
-                b = ob;
-                pa = oa;
+    for (int o = LANES / 2; o > 0; o >>= 1) {
+        const int ob = __shfl_xor_sync(0xffffffffu, b, o);
+        const float oa = __shfl_xor_sync(0xffffffffu, pa, o);
+        if (ob != 0x7fffffff && (b == 0x7fffffff || pair_better(e.amp, ob, oa, b, pa))) {
+            b = ob;
+            pa = oa;
+        }
+    }
+    return b;
+}
+
+// match[a]: the partner of XZ entry a where a is that one's partner too, else -1
+template <int LANES>
+__device__ __forceinline__ void pair_match(const ulm_loc2d* __restrict__ L, int n, int F, int S, int P,
+                                           const int* __restrict__ poff, int* __restrict__ match)
+{
+    constexpr int PER = 256 / LANES;
+    for (int a0 = blockIdx.x * PER; a0 < n; a0 += gridDim.x * PER) {
+        const int a = a0 + threadIdx.x / LANES;
+        ulm_loc2d x{}, y{};
+        if (a < n) x = L[a];
+        const bool xz = a < n && x.axis == 0;
+        int m = -1;
+        if (__any_sync(0xffffffffu, xz)) {
+            const int b = pair_search<LANES>(L, n, x, xz, F, S, P, poff);
+            const bool found = b != 0x7fffffff;
+            if (__any_sync(0xffffffffu, found)) {
+                if (found) y = L[b];
+                if (pair_search<LANES>(L, n, y, found, F, S, P, poff) == a) m = b;
             }
         }
-        if (a < n && sub == 0) best[a] = b == 0x7fffffff ? -1 : b;
+        if (a < n && threadIdx.x % LANES == 0) match[a] = m;
     }
 }
 
-// entry a is the XZ half of a match
-__device__ __forceinline__ bool pair_mutual(const ulm_loc2d* __restrict__ L, const int* __restrict__ best, int a)
+// Matches of a list: every XZ entry searches its partner, and that one back.  Sixteen
+// lanes share an entry (with one, a serial chain of loads and FP64 divisions, 2 392
+// entries took 53 us, now 13) until the entries alone fill the chip, then two: 270 570 entries of the paper's ensemble 267 us with one lane, 104 with sixteen, 86
+// with eight, 80 with two; 41 226 of a small geometry 114, 29, 30 and 50.  (Searches from
+// both axes, so that none follows another, do twice the tests where few entries have a
+// partner: 537 122 entries of which 820 match took 195 us; one lane 132, two 101.)
+// Times of ulm_pair3d.
+#define PAIR_LANES 16
+#define PAIR_WIDE (1 << 18)   // entries from which on two lanes share one
+__global__ void __launch_bounds__(256) k_pair_match(const ulm_loc2d* __restrict__ L, const int* __restrict__ n2d, int cap2d,
+                                                    int F, int S, int P, const int* __restrict__ poff, int* __restrict__ match)
 {
-    const int b = best[a];
-    return b >= 0 && L[a].axis == 0 && best[b] == a;
+    grid_wait();
+    const int n = min(*n2d, cap2d);
+    if (n < PAIR_WIDE) pair_match<PAIR_LANES>(L, n, F, S, P, poff, match);
+    else pair_match<2>(L, n, F, S, P, poff, match);
 }
 
 #define PAIR_CHUNK 1024   // list entries whose matches are counted together
 
-__global__ void __launch_bounds__(256) k_pair_count(const ulm_loc2d* __restrict__ L, const int* __restrict__ n2d, int cap2d,
-                                                    const int* __restrict__ best, int* __restrict__ part)
+__global__ void __launch_bounds__(256) k_pair_count(const int* __restrict__ n2d, int cap2d, const int* __restrict__ match,
+                                                    int* __restrict__ part)
 {
     grid_wait();
     __shared__ int red[8];
@@ -874,7 +896,7 @@ __global__ void __launch_bounds__(256) k_pair_count(const ulm_loc2d* __restrict_
 #pragma unroll
         for (int q = 0; q < PAIR_CHUNK; q += 256) {
             const int a = c * PAIR_CHUNK + q + threadIdx.x;
-            if (a < n && pair_mutual(L, best, a)) ++m;
+            if (a < n && match[a] >= 0) ++m;
         }
         m = __reduce_add_sync(0xffffffffu, m);
         __syncthreads();
@@ -889,7 +911,7 @@ __global__ void __launch_bounds__(256) k_pair_count(const ulm_loc2d* __restrict_
 }
 
 __global__ void __launch_bounds__(256) k_pair_write(const ulm_loc2d* __restrict__ L, const int* __restrict__ n2d, int cap2d,
-                                                    const int* __restrict__ best, const int* __restrict__ part,
+                                                    const int* __restrict__ match, const int* __restrict__ part,
                                                     ulm_loc3d* __restrict__ out, int cap3d, int* __restrict__ n3d,
                                                     unsigned* __restrict__ status)
 {
@@ -906,12 +928,12 @@ __global__ void __launch_bounds__(256) k_pair_write(const ulm_loc2d* __restrict_
         unsigned m = 0u;
 #pragma unroll
         for (int q = 0; q < PER; ++q)
-            if (a0 + q < n && pair_mutual(L, best, a0 + q)) m |= 1u << q;
+            if (a0 + q < n && match[a0 + q] >= 0) m |= 1u << q;
         int all;
         int dst = block_offset(part, c, __popc(m), red, &all);
         if (threadIdx.x == 0 && (c + 1) * PAIR_CHUNK >= n) *n3d = all;
         while (m) {
-            const int a = a0 + __ffs(m) - 1, b = best[a];
+            const int a = a0 + __ffs(m) - 1, b = match[a];
             m &= m - 1;
             if (dst >= cap3d) {
                 atomicOr(status, ST_CAPACITY);
@@ -975,9 +997,9 @@ static rca_status slots_gather(rca_handle* h, const Slots& o, int nslots, int ns
     return cuda_check(h, cudaGetLastError(), "gather kernel");
 }
 
-// pairing on scratch: best [cap2d], part [chunks of PAIR_CHUNK]
+// pairing on scratch: match [cap2d], part [chunks of PAIR_CHUNK]
 static rca_status pair_launch(rca_handle* h, const GeomDev& g, const ulm_loc2d* L, const int* n2d, int cap2d, int F,
-                              const int* poff, int* best, int* part, ulm_loc3d* out, int cap3d, int* n3d)
+                              const int* poff, int* match, int* part, ulm_loc3d* out, int cap3d, int* n3d)
 {
     const int nn = std::max(cap2d, 1);
     if (nn > SCAN_MAX) return set_error(h, RCA_ERR_UNSUPPORTED, "scan over more than %d entries", SCAN_MAX);
@@ -988,9 +1010,9 @@ static rca_status pair_launch(rca_handle* h, const GeomDev& g, const ulm_loc2d* 
     const int cap_blocks = 16 * sms;
     const int nb = std::min(cap_blocks, (nn + 256 / PAIR_LANES - 1) / (256 / PAIR_LANES));
     const int nc = std::min(cap_blocks, (nn + PAIR_CHUNK - 1) / PAIR_CHUNK);
-    launch_chain(k_pair_best, dim3(nb), dim3(256), 0, h->stream, L, n2d, cap2d, F, g.S, g.P, poff, best);
-    launch_chain(k_pair_count, dim3(nc), dim3(256), 0, h->stream, L, n2d, cap2d, best, part);
-    launch_chain(k_pair_write, dim3(nc), dim3(256), 0, h->stream, L, n2d, cap2d, best, part, out, cap3d, n3d, h->d_status);
+    launch_chain(k_pair_match, dim3(nb), dim3(256), 0, h->stream, L, n2d, cap2d, F, g.S, g.P, poff, match);
+    launch_chain(k_pair_count, dim3(nc), dim3(256), 0, h->stream, n2d, cap2d, match, part);
+    launch_chain(k_pair_write, dim3(nc), dim3(256), 0, h->stream, L, n2d, cap2d, match, part, out, cap3d, n3d, h->d_status);
     return cuda_check(h, cudaGetLastError(), "pair kernels");
 }
 
@@ -1114,8 +1136,8 @@ rca_status launch_pair3d(rca_handle* h, const rca_tables* t, const ulm_loc2d* L,
     const int nplanes = F * 2 * g.S;
     rca_status st = RCA_OK;
     const int nn = std::max(cap2d, 1);
-    int* best = (int*)ws_get(h, WS_FLAGS, (size_t)nn * sizeof(int), &st);
-    if (!best) return st;
+    int* match = (int*)ws_get(h, WS_FLAGS, (size_t)nn * sizeof(int), &st);
+    if (!match) return st;
     int* part = (int*)ws_get(h, WS_MISC, (size_t)((nn + PAIR_CHUNK - 1) / PAIR_CHUNK) * sizeof(int), &st);
     if (!part) return st;
     if (!plane_off) {
@@ -1124,7 +1146,7 @@ rca_status launch_pair3d(rca_handle* h, const rca_tables* t, const ulm_loc2d* L,
         launch_chain(k_list_plane_offsets, dim3((nplanes + 1 + 255) / 256), dim3(256), 0, h->stream, L, n2d, cap2d, g.S, nplanes, poff);
         plane_off = poff;
     }
-    return pair_launch(h, g, L, n2d, cap2d, F, plane_off, best, part, out, cap3d, n3d);
+    return pair_launch(h, g, L, n2d, cap2d, F, plane_off, match, part, out, cap3d, n3d);
 }
 
 // detection and pairing of one ensemble: the detection's gather writes the plane
@@ -1157,7 +1179,7 @@ rca_status launch_detect_pair(rca_handle* h, const rca_tables* t, const float* A
 // process (a device reset makes the kept address stale; rca.h says so).
 //
 // Nothing in it needs clearing between calls: each call writes every entry
-// it reads (plane offsets for all planes, partners for all live entries, one
+// it reads (plane offsets for all planes, matches for all live entries, one
 // count per live chunk), so the previous call's contents are never seen.
 // ---------------------------------------------------------------------------
 namespace {
@@ -1165,8 +1187,8 @@ namespace {
 constexpr size_t na_round(size_t b) { return (b + 255) & ~(size_t)255; }
 constexpr int NA_CHUNKS = (ULM_PAIR3D_NOALLOC_MAX_2D + PAIR_CHUNK - 1) / PAIR_CHUNK;
 constexpr size_t NA_POFF = 0;
-constexpr size_t NA_BEST = NA_POFF + na_round((size_t)(ULM_PAIR3D_NOALLOC_MAX_PLANES + 1) * sizeof(int));
-constexpr size_t NA_PART = NA_BEST + na_round((size_t)ULM_PAIR3D_NOALLOC_MAX_2D * sizeof(int));
+constexpr size_t NA_MATCH = NA_POFF + na_round((size_t)(ULM_PAIR3D_NOALLOC_MAX_PLANES + 1) * sizeof(int));
+constexpr size_t NA_PART = NA_MATCH + na_round((size_t)ULM_PAIR3D_NOALLOC_MAX_2D * sizeof(int));
 constexpr size_t NA_BYTES = ULM_PAIR3D_NOALLOC_SCRATCH_BYTES;   // the size that rca.h states
 static_assert(NA_PART + na_round((size_t)NA_CHUNKS * sizeof(int)) <= NA_BYTES, "scratch size stated in rca.h is too small");
 
@@ -1211,11 +1233,11 @@ rca_status launch_pair3d_noalloc(rca_handle* h, const rca_tables* t, const ulm_l
     rca_status st = pair_scratch(h, &base);
     if (st != RCA_OK) return st;
     int* poff = reinterpret_cast<int*>(base + NA_POFF);
-    int* best = reinterpret_cast<int*>(base + NA_BEST);
+    int* match = reinterpret_cast<int*>(base + NA_MATCH);
     int* part = reinterpret_cast<int*>(base + NA_PART);
     const int np = (int)nplanes;
     launch_chain(k_list_plane_offsets, dim3((np + 1 + 255) / 256), dim3(256), 0, h->stream, L, n2d, cap2d, g.S, np, poff);
-    return pair_launch(h, g, L, n2d, cap2d, F, poff, best, part, out, cap3d, n3d);
+    return pair_launch(h, g, L, n2d, cap2d, F, poff, match, part, out, cap3d, n3d);
 }
 
 rca_status launch_detect_map(rca_handle* h, const rca_tables* t, const float* map, int up, const float* A, const float* M,

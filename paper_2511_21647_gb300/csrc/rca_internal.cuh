@@ -45,7 +45,7 @@ enum WsSlot {
     WS_CAND,       // ulm_loc2d [strips][CAND_CAP]
     WS_CANDCNT,    // candidate totals and counts (slots_bytes)
     WS_PLANEOFF,   // int [planes + 1]
-    WS_FLAGS,      // pairing partner of every list entry
+    WS_FLAGS,      // pairing match of every list entry
     WS_MISC,       // small scratch
     WS_TRACK,      // tracking: frame offsets, links, flags, positions, per-localisation tracks
     WS_MOTION,     // motion estimation: twiddles, row spectra, reference spectrum, correlations
