@@ -57,19 +57,41 @@ __host__ __device__ constexpr int wr_off(int R)
     return R == 8 ? 0 : R == 12 ? 8 : R == 16 ? 20 : R == 20 ? 36 : -1;
 }
 
-// complex sums, differences and real multiples as packed pairs: one issue slot instead of two, the same rounding
-__device__ __forceinline__ uint64_t f2p(float2 a) { return f2_pack(a.x, a.y); }
-__device__ __forceinline__ float2 f2add(float2 a, float2 b) { return f2_unpack(f2_add(f2p(a), f2p(b))); }
-__device__ __forceinline__ float2 f2sub(float2 a, float2 b) { return f2_unpack(f2_sub(f2p(a), f2p(b))); }
-__device__ __forceinline__ float2 f2scale(float2 a, float s) { return f2_unpack(f2_mul(f2p(a), f2_pack(s, s))); }
-__device__ __forceinline__ float2 f2fma(float2 a, float s, float2 b) { return f2_unpack(f2_fma(f2p(a), f2_pack(s, s), f2p(b))); }
+// complex sums, differences and real multiples.  PK: as packed pairs, one issue slot instead of two, the same rounding;
+// else scalar: k_separate's largest form, one CTA of eight warps an SM, waits for results rather than for issue slots
+// (60 rows of 512 frames, 32 elements, six subsets: 648 us packed, 613 scalar)
+template <bool PK>
+__device__ __forceinline__ float2 f2add(float2 a, float2 b)
+{
+    if constexpr (PK) return f2_unpack(f2_add(f2_pack(a.x, a.y), f2_pack(b.x, b.y)));
+    else return make_float2(a.x + b.x, a.y + b.y);
+}
+template <bool PK>
+__device__ __forceinline__ float2 f2sub(float2 a, float2 b)
+{
+    if constexpr (PK) return f2_unpack(f2_sub(f2_pack(a.x, a.y), f2_pack(b.x, b.y)));
+    else return make_float2(a.x - b.x, a.y - b.y);
+}
+template <bool PK>
+__device__ __forceinline__ float2 f2scale(float2 a, float s)
+{
+    if constexpr (PK) return f2_unpack(f2_mul(f2_pack(a.x, a.y), f2_pack(s, s)));
+    else return make_float2(a.x * s, a.y * s);
+}
+template <bool PK>
+__device__ __forceinline__ float2 f2fma(float2 a, float s, float2 b)
+{
+    if constexpr (PK) return f2_unpack(f2_fma(f2_pack(a.x, a.y), f2_pack(s, s), f2_pack(b.x, b.y)));
+    else return make_float2(fmaf(a.x, s, b.x), fmaf(a.y, s, b.y));
+}
 // a + i^e b, e known at compile time; the odd quarter turns in scalar operations, whose operands need no swap
+template <bool PK>
 __device__ __forceinline__ float2 addq(float2 a, float2 b, int e)
 {
     e &= 3;
-    return e == 0   ? f2add(a, b)
+    return e == 0   ? f2add<PK>(a, b)
            : e == 1 ? make_float2(a.x - b.y, a.y + b.x)
-           : e == 2 ? f2sub(a, b)
+           : e == 2 ? f2sub<PK>(a, b)
                     : make_float2(a.x + b.y, a.y - b.x);
 }
 // a w (forward) or a conj(w) (inverse)
@@ -93,74 +115,74 @@ __device__ __forceinline__ float sqrt_approx(float x)
     return r;
 }
 // R-point DFT in registers, y_k = sum_n x_n exp(-+2 pi i n k / R)
-template <int R, bool INV> struct Dft;
+template <int R, bool INV, bool PK> struct Dft;
 
-template <bool INV> struct Dft<2, INV> {
+template <bool INV, bool PK> struct Dft<2, INV, PK> {
     static __device__ __forceinline__ void run(float2 (&v)[2], const SepConst&)
     {
         const float2 a = v[0];
-        v[0] = f2add(a, v[1]);
-        v[1] = f2sub(a, v[1]);
+        v[0] = f2add<PK>(a, v[1]);
+        v[1] = f2sub<PK>(a, v[1]);
     }
 };
 
 // from the sum and difference of inputs 1 and 2, st t and sd d with signs known at compile time
-template <bool INV>
+template <bool INV, bool PK>
 __device__ __forceinline__ void core3(float2 (&v)[3], float2 t, float2 d, float st, int sd, const SepConst& c)
 {
-    const float2 m = f2fma(t, -0.5f * st, v[0]);
+    const float2 m = f2fma<PK>(t, -0.5f * st, v[0]);
     const float k = INV == (sd > 0) ? c.s3 : -c.s3;                            // v1, v2 = m +- i k d
-    v[0] = st > 0.f ? f2add(v[0], t) : f2sub(v[0], t);
+    v[0] = st > 0.f ? f2add<PK>(v[0], t) : f2sub<PK>(v[0], t);
     v[1] = make_float2(fmaf(-k, d.y, m.x), fmaf(k, d.x, m.y));
     v[2] = make_float2(fmaf(k, d.y, m.x), fmaf(-k, d.x, m.y));
 }
 
-template <bool INV> struct Dft<3, INV> {
+template <bool INV, bool PK> struct Dft<3, INV, PK> {
     static __device__ __forceinline__ void run(float2 (&v)[3], const SepConst& c)
     {
-        core3<INV>(v, f2add(v[1], v[2]), f2sub(v[1], v[2]), 1.f, 1, c);
+        core3<INV, PK>(v, f2add<PK>(v[1], v[2]), f2sub<PK>(v[1], v[2]), 1.f, 1, c);
     }
 };
 
-template <bool INV> struct Dft<4, INV> {
+template <bool INV, bool PK> struct Dft<4, INV, PK> {
     static __device__ __forceinline__ void run(float2 (&v)[4], const SepConst&)
     {
-        const float2 t0 = f2add(v[0], v[2]), t1 = f2sub(v[0], v[2]);
-        const float2 t2 = f2add(v[1], v[3]), t3 = f2sub(v[1], v[3]);
-        v[0] = f2add(t0, t2);
-        v[2] = f2sub(t0, t2);
-        v[1] = addq(t1, t3, INV ? 1 : 3);
-        v[3] = addq(t1, t3, INV ? 3 : 1);
+        const float2 t0 = f2add<PK>(v[0], v[2]), t1 = f2sub<PK>(v[0], v[2]);
+        const float2 t2 = f2add<PK>(v[1], v[3]), t3 = f2sub<PK>(v[1], v[3]);
+        v[0] = f2add<PK>(t0, t2);
+        v[2] = f2sub<PK>(t0, t2);
+        v[1] = addq<PK>(t1, t3, INV ? 1 : 3);
+        v[3] = addq<PK>(t1, t3, INV ? 3 : 1);
     }
 };
 
 // from the sums and differences of inputs 1, 4 (a1, s1 b1) and 2, 3 (a2, b2), s1 = +-1 known at compile time
-template <bool INV>
+template <bool INV, bool PK>
 __device__ __forceinline__ void core5(float2 (&v)[5], float2 a1, float2 b1, float2 a2, float2 b2, int s1, const SepConst& c)
 {
-    const float2 m1 = f2fma(a2, c.c52, f2fma(a1, c.c51, v[0]));
-    const float2 m2 = f2fma(a2, c.c51, f2fma(a1, c.c52, v[0]));
-    const float2 r1 = s1 > 0 ? f2fma(b2, c.s52, f2scale(b1, c.s51)) : f2fma(b1, -c.s51, f2scale(b2, c.s52));
-    const float2 r2 = s1 > 0 ? f2fma(b2, -c.s51, f2scale(b1, c.s52)) : f2fma(b1, c.s52, f2scale(b2, c.s51));   // s1 r2
+    const float2 m1 = f2fma<PK>(a2, c.c52, f2fma<PK>(a1, c.c51, v[0]));
+    const float2 m2 = f2fma<PK>(a2, c.c51, f2fma<PK>(a1, c.c52, v[0]));
+    const float2 r1 = s1 > 0 ? f2fma<PK>(b2, c.s52, f2scale<PK>(b1, c.s51)) : f2fma<PK>(b1, -c.s51, f2scale<PK>(b2, c.s52));
+    const float2 r2 = s1 > 0 ? f2fma<PK>(b2, -c.s51, f2scale<PK>(b1, c.s52)) : f2fma<PK>(b1, c.s52, f2scale<PK>(b2, c.s51));   // s1 r2
     const int e1 = INV ? 1 : 3, e2 = e1 + (s1 > 0 ? 0 : 2);
-    v[0] = f2add(v[0], f2add(a1, a2));
-    v[1] = addq(m1, r1, e1);
-    v[4] = addq(m1, r1, e1 + 2);
-    v[2] = addq(m2, r2, e2);
-    v[3] = addq(m2, r2, e2 + 2);
+    v[0] = f2add<PK>(v[0], f2add<PK>(a1, a2));
+    v[1] = addq<PK>(m1, r1, e1);
+    v[4] = addq<PK>(m1, r1, e1 + 2);
+    v[2] = addq<PK>(m2, r2, e2);
+    v[3] = addq<PK>(m2, r2, e2 + 2);
 }
 
-template <bool INV> struct Dft<5, INV> {
+template <bool INV, bool PK> struct Dft<5, INV, PK> {
     static __device__ __forceinline__ void run(float2 (&v)[5], const SepConst& c)
     {
-        core5<INV>(v, f2add(v[1], v[4]), f2sub(v[1], v[4]), f2add(v[2], v[3]), f2sub(v[2], v[3]), 1, c);
+        core5<INV, PK>(v, f2add<PK>(v[1], v[4]), f2sub<PK>(v[1], v[4]), f2add<PK>(v[2], v[3]), f2sub<PK>(v[2], v[3]), 1, c);
     }
 };
 
 // R = R1 R2 by one Cooley-Tukey split in registers: n = R2 n1 + n2,
 // k = k1 + R1 k2; the inner twiddles W_R^(n2 k1) are kernel-parameter
 // constants at compile-time offsets.
-template <int R1, int R2, bool INV> struct DftC {
+template <int R1, int R2, bool INV, bool PK> struct DftC {
     static __device__ __forceinline__ void run(float2 (&v)[R1 * R2], const SepConst& c)
     {
         constexpr int W0 = wr_off(R1 * R2);
@@ -169,7 +191,7 @@ template <int R1, int R2, bool INV> struct DftC {
             float2 a[R1];
 #pragma unroll
             for (int n1 = 0; n1 < R1; ++n1) a[n1] = v[R2 * n1 + n2];
-            Dft<R1, INV>::run(a, c);
+            Dft<R1, INV, PK>::run(a, c);
 #pragma unroll
             for (int k1 = 0; k1 < R1; ++k1)
                 v[R2 * k1 + n2] = (n2 * k1 == 0) ? a[k1] : twmul<INV>(a[k1], c.wr[W0 + n2 * k1]);
@@ -180,7 +202,7 @@ template <int R1, int R2, bool INV> struct DftC {
             float2 b[R2];
 #pragma unroll
             for (int n2 = 0; n2 < R2; ++n2) b[n2] = v[R2 * k1 + n2];
-            Dft<R2, INV>::run(b, c);
+            Dft<R2, INV, PK>::run(b, c);
 #pragma unroll
             for (int k2 = 0; k2 < R2; ++k2) o[k1 + R1 * k2] = b[k2];
         }
@@ -197,7 +219,7 @@ __host__ __device__ constexpr int crt_unit(int a, int b)      // 1 mod a, 0 mod 
     while (n % a != 1 % a) n += b;
     return n;
 }
-template <int R1, int R2, bool INV> struct DftP {
+template <int R1, int R2, bool INV, bool PK> struct DftP {
     static __device__ __forceinline__ void run(float2 (&v)[R1 * R2], const SepConst& c)
     {
         constexpr int R = R1 * R2, E1 = crt_unit(R1, R2), E2 = crt_unit(R2, R1);
@@ -207,7 +229,7 @@ template <int R1, int R2, bool INV> struct DftP {
             float2 a[R1];
 #pragma unroll
             for (int n1 = 0; n1 < R1; ++n1) a[n1] = v[(E1 * n1 + E2 * n2) % R];
-            Dft<R1, INV>::run(a, c);
+            Dft<R1, INV, PK>::run(a, c);
 #pragma unroll
             for (int k1 = 0; k1 < R1; ++k1) w[R2 * k1 + n2] = a[k1];
         }
@@ -216,21 +238,21 @@ template <int R1, int R2, bool INV> struct DftP {
             float2 b[R2];
 #pragma unroll
             for (int n2 = 0; n2 < R2; ++n2) b[n2] = w[R2 * k1 + n2];
-            Dft<R2, INV>::run(b, c);
+            Dft<R2, INV, PK>::run(b, c);
 #pragma unroll
             for (int k2 = 0; k2 < R2; ++k2) v[(R2 * k1 + R1 * k2) % R] = b[k2];
         }
     }
 };
 
-template <int R, bool INV> struct Radix { using T = Dft<R, INV>; };
-template <bool INV> struct Radix<6, INV> { using T = DftP<2, 3, INV>; };
-template <bool INV> struct Radix<8, INV> { using T = DftC<2, 4, INV>; };
-template <bool INV> struct Radix<10, INV> { using T = DftP<2, 5, INV>; };
-template <bool INV> struct Radix<12, INV> { using T = DftP<4, 3, INV>; };
-template <bool INV> struct Radix<15, INV> { using T = DftP<3, 5, INV>; };
-template <bool INV> struct Radix<16, INV> { using T = DftC<4, 4, INV>; };
-template <bool INV> struct Radix<20, INV> { using T = DftP<4, 5, INV>; };
+template <int R, bool INV, bool PK> struct Radix { using T = Dft<R, INV, PK>; };
+template <bool INV, bool PK> struct Radix<6, INV, PK> { using T = DftP<2, 3, INV, PK>; };
+template <bool INV, bool PK> struct Radix<8, INV, PK> { using T = DftC<2, 4, INV, PK>; };
+template <bool INV, bool PK> struct Radix<10, INV, PK> { using T = DftP<2, 5, INV, PK>; };
+template <bool INV, bool PK> struct Radix<12, INV, PK> { using T = DftP<4, 3, INV, PK>; };
+template <bool INV, bool PK> struct Radix<15, INV, PK> { using T = DftP<3, 5, INV, PK>; };
+template <bool INV, bool PK> struct Radix<16, INV, PK> { using T = DftC<4, 4, INV, PK>; };
+template <bool INV, bool PK> struct Radix<20, INV, PK> { using T = DftP<4, 5, INV, PK>; };
 
 // twiddle-table row pitch of a radix-R pass (R - 1 entries, even for 16-byte pairs)
 __host__ __device__ constexpr int tw_pitch(int R) { return (R - 1 + 1) & ~1; }
@@ -239,7 +261,7 @@ __host__ __device__ constexpr int tw_pitch(int R) { return (R - 1 + 1) & ~1; }
 // radices before this one (product Ns), butterfly idx (k = idx mod Ns) takes
 // in[idx + r F / R], twiddles them by W_F^(k r F / (Ns R)) = T[k pitch + r - 1],
 // transforms and stores output u at (idx - k) R + k + u Ns.
-template <int R, bool INV>
+template <int R, bool INV, bool PK>
 __device__ __forceinline__ void sp_pass(const float2* __restrict__ in, float2* __restrict__ out, int F, int Ns,
                                         const float2* __restrict__ T, const SepConst& c)
 {
@@ -261,7 +283,7 @@ __device__ __forceinline__ void sp_pass(const float2* __restrict__ in, float2* _
                 if (r + 1 < R) v[r + 1] = twmul<INV>(v[r + 1], make_float2(w.z, w.w));
             }
         }
-        Radix<R, INV>::T::run(v, c);
+        Radix<R, INV, PK>::T::run(v, c);
         float2* dst = out + ((idx - k) * R + k) * SP_G + g;
 #pragma unroll
         for (int u = 0; u < R; ++u) dst[u * Ns * SP_G] = v[u];
@@ -269,7 +291,7 @@ __device__ __forceinline__ void sp_pass(const float2* __restrict__ in, float2* _
 }
 
 // all passes; returns the buffer that holds the result
-template <bool INV>
+template <bool INV, bool PK>
 __device__ float2* sp_fft(float2* a, float2* b, const SepConst& sc, const float2* tws)
 {
     int Ns = 1;
@@ -278,17 +300,17 @@ __device__ float2* sp_fft(float2* a, float2* b, const SepConst& sc, const float2
         const int R = sc.radix[p];
         const float2* T = tws + sc.twoff[p];
         switch (R) {
-            case 2: sp_pass<2, INV>(a, b, F, Ns, T, sc); break;
-            case 3: sp_pass<3, INV>(a, b, F, Ns, T, sc); break;
-            case 4: sp_pass<4, INV>(a, b, F, Ns, T, sc); break;
-            case 5: sp_pass<5, INV>(a, b, F, Ns, T, sc); break;
-            case 6: sp_pass<6, INV>(a, b, F, Ns, T, sc); break;
-            case 8: sp_pass<8, INV>(a, b, F, Ns, T, sc); break;
-            case 10: sp_pass<10, INV>(a, b, F, Ns, T, sc); break;
-            case 12: sp_pass<12, INV>(a, b, F, Ns, T, sc); break;
-            case 15: sp_pass<15, INV>(a, b, F, Ns, T, sc); break;
-            case 16: sp_pass<16, INV>(a, b, F, Ns, T, sc); break;
-            default: sp_pass<20, INV>(a, b, F, Ns, T, sc); break;
+            case 2: sp_pass<2, INV, PK>(a, b, F, Ns, T, sc); break;
+            case 3: sp_pass<3, INV, PK>(a, b, F, Ns, T, sc); break;
+            case 4: sp_pass<4, INV, PK>(a, b, F, Ns, T, sc); break;
+            case 5: sp_pass<5, INV, PK>(a, b, F, Ns, T, sc); break;
+            case 6: sp_pass<6, INV, PK>(a, b, F, Ns, T, sc); break;
+            case 8: sp_pass<8, INV, PK>(a, b, F, Ns, T, sc); break;
+            case 10: sp_pass<10, INV, PK>(a, b, F, Ns, T, sc); break;
+            case 12: sp_pass<12, INV, PK>(a, b, F, Ns, T, sc); break;
+            case 15: sp_pass<15, INV, PK>(a, b, F, Ns, T, sc); break;
+            case 16: sp_pass<16, INV, PK>(a, b, F, Ns, T, sc); break;
+            default: sp_pass<20, INV, PK>(a, b, F, Ns, T, sc); break;
         }
         __syncthreads();
         float2* t = a;
@@ -306,6 +328,7 @@ __global__ void __launch_bounds__(SP_THREADS, MX <= 19 ? 2 : 1)
     k_separate(const void* __restrict__ planes, int pt, const __grid_constant__ SepConst sc, int S, int nz, int N,
                float2* __restrict__ sub, float* __restrict__ A, unsigned* __restrict__ M)
 {
+    constexpr bool PK = MX <= 19;
     extern __shared__ __align__(16) float2 smem[];
     const int F = sc.F, nsub = sc.nsub;
     float2* B0 = smem;
@@ -370,7 +393,7 @@ __global__ void __launch_bounds__(SP_THREADS, MX <= 19 ? 2 : 1)
         __syncthreads();
         // each thread keeps the spectrum's elements threadIdx.x + m SP_THREADS; per subset the masked spectrum is written
         // back for the inverse transform
-        const float2* X = sp_fft<false>(B0, B1, sc, tws);
+        const float2* X = sp_fft<false, PK>(B0, B1, sc, tws);
 #pragma unroll
         for (int m = 0; m < MX; ++m) {
             const int e = threadIdx.x + m * SP_THREADS;
@@ -382,10 +405,10 @@ __global__ void __launch_bounds__(SP_THREADS, MX <= 19 ? 2 : 1)
 #pragma unroll
             for (int m = 0; m < MX; ++m) {
                 const int e = threadIdx.x + m * SP_THREADS;
-                if (e < n_el) B0[e] = sbin[e / SP_G] == s ? f2scale(xr[m], invF) : make_float2(0.f, 0.f);
+                if (e < n_el) B0[e] = sbin[e / SP_G] == s ? f2scale<PK>(xr[m], invF) : make_float2(0.f, 0.f);
             }
             __syncthreads();
-            const float2* Y = sp_fft<true>(B0, B1, sc, tws);
+            const float2* Y = sp_fft<true, PK>(B0, B1, sc, tws);
             if (OUT == SP_OUT_COMPLEX) {
                 float2* dst = sub + (size_t)s * F * 4 * per_axis;
                 for (int i = threadIdx.x; i < n_el; i += SP_THREADS) {
@@ -485,25 +508,25 @@ __device__ __forceinline__ void win_idft(const float2 (&x)[NW * Q], const SepCon
         float2 b[Q];
         // b[m] = i^(m k1) z[m] (Q = 3, 5); z[m] = x[m] + i^(Q k1) x[m + Q]
 #pragma unroll
-        for (int m = 0; m < Q; ++m) b[m] = NW == 1 ? x[m] : addq(x[m], x[(NW - 1) * Q + m], (Q == 4 ? 1 : Q) * k1);
+        for (int m = 0; m < Q; ++m) b[m] = NW == 1 ? x[m] : addq<true>(x[m], x[(NW - 1) * Q + m], (Q == 4 ? 1 : Q) * k1);
         if constexpr (Q == 5) {
             // inputs 1, 4: i^k1 z1 and z4; inputs 2, 3: i^(2 k1) (z2 + i^k1 z3), i^(2 k1) = -1 for odd k1
-            const float2 a1 = addq(b[4], b[1], k1), n1 = addq(b[4], b[1], k1 + 2);      // n1 = -(i^k1 z1 - z4)
-            float2 a2 = addq(b[2], b[3], k1), b2 = addq(b[2], b[3], k1 + 2);
+            const float2 a1 = addq<true>(b[4], b[1], k1), n1 = addq<true>(b[4], b[1], k1 + 2);      // n1 = -(i^k1 z1 - z4)
+            float2 a2 = addq<true>(b[2], b[3], k1), b2 = addq<true>(b[2], b[3], k1 + 2);
             if (k1 & 1) {
                 a2 = make_float2(-a2.x, -a2.y);
                 b2 = make_float2(-b2.x, -b2.y);
             }
-            core5<true>(b, a1, n1, a2, b2, -1, c);
+            core5<true, true>(b, a1, n1, a2, b2, -1, c);
         } else if constexpr (Q == 3) {
             // input 2: i^(2 k1) z2 = s z2, s = +-1; input 1: i^k1 z1 = s i^(-k1) z1
-            const float2 t = addq(b[2], b[1], -k1), d = addq(b[2], b[1], 2 - k1);
-            core3<true>(b, t, d, k1 & 1 ? -1.f : 1.f, k1 & 1 ? 1 : -1, c);
+            const float2 t = addq<true>(b[2], b[1], -k1), d = addq<true>(b[2], b[1], 2 - k1);
+            core3<true, true>(b, t, d, k1 & 1 ? -1.f : 1.f, k1 & 1 ? 1 : -1, c);
         } else {
 #pragma unroll
             for (int m = 1; m < Q; ++m)
                 if (k1) b[m] = twmul<true>(b[m], c.wr[wr_off(16) + m * k1]);
-            Dft<Q, true>::run(b, c);
+            Dft<Q, true, true>::run(b, c);
         }
 #pragma unroll
         for (int k2 = 0; k2 < Q; ++k2) store(Q == 4 ? k1 + 4 * k2 : (Q * k1 + 4 * k2) % (4 * Q), b[k2]);
@@ -543,7 +566,7 @@ __device__ __forceinline__ void win_pass2(float2 (&v)[R2], const float2* B, cons
         v[r] = twmul<INV>(v[r], make_float2(w.x, w.y));
         if (r + 1 < R2) v[r + 1] = twmul<INV>(v[r + 1], make_float2(w.z, w.w));
     }
-    Radix<R2, INV>::T::run(v, c);
+    Radix<R2, INV, true>::T::run(v, c);
 }
 
 // amplitudes of one subset from its frames Y [F][SP_G]: thread (lateral pixel l, chunk of PER frames); the frame maxima
@@ -660,7 +683,7 @@ __global__ void __launch_bounds__(R1* SP_G, R1 == 20 ? 2 : R1 == 16 ? 3 : 4)
 #pragma unroll
                 for (int r = 0; r < R1; ++r) v[r] = load_c(w + r, 0, pt);
             }
-            Radix<R1, false>::T::run(v, sc);
+            Radix<R1, false, true>::T::run(v, sc);
             float2* dst = X + idx * R1 * SP_G + g;
 #pragma unroll
             for (int u = 0; u < R1; ++u) dst[u * SP_G] = v[u];
@@ -671,7 +694,7 @@ __global__ void __launch_bounds__(R1* SP_G, R1 == 20 ? 2 : R1 == 16 ? 3 : 4)
             float2 v[RR];
             win_pass2<R1, RR, false>(v, X, tws, sc);
 #pragma unroll
-            for (int u = 0; u < RR; ++u) X[threadIdx.x + u * NT] = f2scale(v[u], invF);
+            for (int u = 0; u < RR; ++u) X[threadIdx.x + u * NT] = f2scale<true>(v[u], invF);
         };
         auto subset = [&](auto r2, int s) {
             constexpr int RR = decltype(r2)::value;
