@@ -867,8 +867,9 @@ __device__ __forceinline__ void pair_match(const ulm_loc2d* __restrict__ L, int 
 
 // Matches of a list: every XZ entry searches its partner, and that one back.  Sixteen
 // lanes share an entry (with one, a serial chain of loads and FP64 divisions, 2 392
-// entries took 53 us, now 13) until the entries alone fill the chip, then two: 270 570 entries of the paper's ensemble 267 us with one lane, 104 with sixteen, 86
-// with eight, 80 with two; 41 226 of a small geometry 114, 29, 30 and 50.  (Searches from
+// entries took 53 us, now 13) until the entries alone fill the chip, then two: 270 570
+// entries of the paper's ensemble 267 us with one lane, 104 with sixteen, 86 with
+// eight, 80 with two; 41 226 of a small geometry 114, 29, 30 and 50.  (Searches from
 // both axes, so that none follows another, do twice the tests where few entries have a
 // partner: 537 122 entries of which 820 match took 195 us; one lane 132, two 101.)
 // Times of ulm_pair3d.
