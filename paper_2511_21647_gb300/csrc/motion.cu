@@ -20,8 +20,9 @@
 // x, registers along z): the pointwise product and the inverse take it as it is.
 // Frames go through in chunks whose spectra stay in the L2 cache, so that HBM sees
 // the slices once.  300 frames of the paper's slices: 4.5 ms with radix-4 passes in
-// shared memory (rows 0.92, columns 2.43, peak 1.15) and 64-frame chunks; now 1.77
-// (chunks of 32 MB: 2.30, too few CTAs per launch; of 96 MB: 1.99, past the L2).
+// shared memory (rows 0.92, columns 2.43, peak 1.15) and 64-frame chunks; 1.77 with these
+// kernels, 1.66 with dependent launches (chunks of 32 MB: 2.30, too few CTAs per
+// launch; of 96 MB: 1.99, past the L2; both without those).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>

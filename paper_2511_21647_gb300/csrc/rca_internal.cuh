@@ -158,8 +158,8 @@ struct rca_tables {
 // a row group is one run; otherwise (split) N / 32 warps hold the pairs twice,
 // the second half for the next run of rows, so that one broadcast record still
 // serves two pixels of every lane.  Unpaired: one pixel per lane, LW = ceil(N / 32).
-// (45 frames of 96 elements: Stage 1 553 us unpaired, 503 split; 6548 frames of 32
-// elements in a batch: 4.33 and 3.95 ms.)
+// (45 frames of 96 elements: Stage 1 553 us unpaired, 503 split; a batch of 5259 frames
+// of 32 elements, 20854 (frame, transmission) pairs: 4.33 and 3.95 ms.)
 enum { S1_UNPAIRED = 0, S1_PAIRED = 1, S1_SPLIT = 2 };
 struct S1Layout {
     int LW, RG, slots, per, pair;
@@ -305,10 +305,12 @@ rca_status launch_pair3d_noalloc(rca_handle* h, const rca_tables* t, const ulm_l
 // one's blocks have left, and grid_wait() holds them until its results are visible.
 // Every kernel so launched calls grid_wait() before it touches global memory, so a
 // chain of them keeps the stream's order; what is hidden is the launch of one
-// behind the tail of the other (beamforming of 8 tiny frames, four kernels: 28.7 us,
-// with it 19.7).  No kernel lets the next one's blocks in any earlier: with
-// griddepcontrol.launch_dependents behind the wait the paper's ensemble took 13.68 ms
-// instead of 13.57, a training step 198 us instead of 192, the tiny chain 20.2 us.
+// behind the tail of the other: beamforming of 8 tiny frames, four kernels, 28.7 us,
+// with it 19.5, for calls queued back to back (the first call of an idle stream has no
+// tail to hide behind and takes 166 us either way).  No kernel lets the next one's
+// blocks in any earlier: with griddepcontrol.launch_dependents behind the wait the
+// paper's ensemble took 13.68 ms instead of 13.57, a training step 198 us instead of
+// 192, the tiny chain 20.2 us.
 // ---------------------------------------------------------------------------
 template <typename... P, typename... A>
 inline cudaError_t launch_chain(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
