@@ -232,7 +232,7 @@ def main():
 
     stages = ["ingest", "stage1", "stage2", "enhance", "detect2d", "pair3d"]
     # kernels per call: mean + demodulation; detect + gather (with its scan);
-    # list offsets + best partners + counts + write
+    # list offsets + matches + counts + write
     launches = {"ingest": 2, "stage1": 1, "stage2": 1, "enhance": 1, "detect2d": 2, "pair3d": 4}
 
     def step(ev=None):

@@ -24,7 +24,8 @@
 // operands (56 cycles at 128 B per clock, against 48 of the tensor pipe; as
 // three MMAs of N = 32 it would read 15 KB), about 1040 cycles per row of 128
 // pixels for the three layers, and the CUDA cores' accesses add about half as
-// much (ncu: 54 % and 29 % of the elapsed cycles).  Two strips per CTA share the
+// much (ncu, 16 frames of the paper's planes: the operand reads 67 % of the elapsed
+// cycles, those accesses 38 %, the tensor pipe 43 %).  Two strips per CTA share the
 // 77 KB of weights and fill each other's waits; 240 of 512 TMEM columns each.
 // Separate warps for the edge layers, the hidden layers and the issue of MMAs
 // keep a step short: one set of four warps that also issued took 5 800 cycles a
